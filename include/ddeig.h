@@ -58,7 +58,7 @@ extern "C" {
 #define DD_EUNSUPPORTED -9  /* option combination not built (e.g. a precision for this size) */
 
 /* Local-inverse precision (the only place below FP64). */
-#define DD_PREC_FP64 0      /* local solves by FP64 banded Cholesky (plain method) */
+#define DD_PREC_FP64 0      /* local solves in FP64 (block elimination; the plain method) */
 #define DD_PREC_TF32 1      /* dense local inverses, TF32 tensor-core GEMM, FP32 accumulate */
 #define DD_PREC_BF16 2      /* dense local inverses, BF16 tensor-core GEMM, FP32 accumulate */
 #define DD_PREC_FP8  3      /* dense local inverses, FP8 (E4M3) tensor-core GEMM, FP32 accumulate;
@@ -137,7 +137,8 @@ int dd_cell_eigenpair(dd_ctx* ctx, double* sigma_out, double* psi_cell_out);
 
 /*
  * dd_coarse_build -- local matrices A_{sigma,i} = R_i A_sigma R_i^T per distinct subdomain
- * type, factorised (FP64 banded Cholesky) and, for TF32/BF16, inverted and rounded; the
+ * type, factorised (FP64: block elimination along x_1 with dense inverse Schur complements;
+ * TF32/BF16: FP32 banded Cholesky, inverted and rounded); the
  * coarse matrix A_{sigma,0} = R_0 A_sigma R_0^T (Sec. 3.1) assembled and factorised.
  * DD_ENOTSPD if a local or coarse matrix is not positive definite.
  */
@@ -365,9 +366,9 @@ int dd_coarse_matrix(dd_ctx* ctx, double* A0_host);
  *   DD_OPT_GEMM_TILE_N  N tile of the mixed local-solve contraction: 128, 160 or 256, 0 = chosen
  *                       by timing each on the context's operands at dd_coarse_build (cached per
  *                       problem shape); the result does not depend on it [0]
- *   DD_OPT_LOCAL_RHS    FP64 local solves: subdomains of one type solved together by one warp,
- *                       1, 2 or 4 (capped by shared memory), 0 = default (2 where allowed) [0]; the result
- *                       does not depend on it (same operations per vector)
+ *   DD_OPT_LOCAL_RHS    FP64 local solves: subdomains of one type solved by one thread block,
+ *                       1, 2 or 4 (capped by the block's size), 0 = chosen by the number of
+ *                       subdomains [0]; the result does not depend on it (same operations per vector)
  *   DD_OPT_FUSED_PQ     p = 1: -1 automatic / 1 one kernel stages p = z + beta p in shared memory
  *                       and applies the stencil from there (one node per thread and pass), 2 the
  *                       same with two nodes per thread and pass (their tap chains interleaved),

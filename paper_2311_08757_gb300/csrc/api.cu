@@ -155,18 +155,6 @@ namespace {
 
 using namespace dd;
 
-// FP64 local solves: groups of up to k consecutive slots of one type, one group per warp
-void set_local_groups(dd_ctx* c, int k) {
-  c->rhs_k = k;
-  c->group_h.clear();
-  for (int t = 0; t < c->ntypes; ++t)
-    for (int j = 0; j < c->type_count[t]; j += k)
-      c->group_h.push_back(make_int2(c->type_first[t] + j, std::min(k, c->type_count[t] - j)));
-  c->ngroups = (int)c->group_h.size();
-  DD_CUDA(cudaMemcpyAsync(c->groups, c->group_h.data(), sizeof(int2) * c->group_h.size(), cudaMemcpyHostToDevice,
-                          c->stream));
-}
-
 void build_subdomains(dd_ctx* c) {
   const Geo& g = c->g;
   int id_of[16];
@@ -182,6 +170,7 @@ void build_subdomains(dd_ctx* c) {
       id_of[key] = c->ntypes;
       c->type_ax[c->ntypes][0] = t1;
       c->type_ax[c->ntypes][1] = t2;
+      c->rep_of_type[c->ntypes] = s;
       ++c->ntypes;
     }
     Sub sb;
@@ -246,7 +235,7 @@ void build_subdomains(dd_ctx* c) {
   c->sub_of_slot = (int*)dev_alloc(c, sizeof(int) * g.nsub);
   c->groups = (int2*)dev_alloc(c, sizeof(int2) * g.nsub);
   DD_CUDA(cudaMemcpyAsync(c->sub_of_slot, sos.data(), sizeof(int) * g.nsub, cudaMemcpyHostToDevice, c->stream));
-  set_local_groups(c, std::min(2, rhs_per_warp(c->nloc_max, c->band)));
+  if (c->grid.precision == DD_PREC_FP64) block_groups(c, 0);
   // p = 1: the prolong-sum computes owners and packed rows in closed form where the formula
   // reproduces these tables exactly (every column, packed row i = subdomain i)
   bool closed = g.p == 1;
@@ -331,9 +320,8 @@ bool use_gemm(const dd_ctx* c) { return c->grid.precision != DD_PREC_FP64; }
 void precond(dd_ctx* c, const double* r, int mode, double* zout = nullptr, bool packed = false) {
   cudaStream_t s = c->stream;
   const bool coarse = c->grid.coarse != 0;
-  double* c0 = coarse ? c->c0 : nullptr;
   if (use_gemm(c)) {
-    if (!packed) TIMED(KC_PACK, s, launch_pack(c, r, c0, s));
+    if (!packed) TIMED(KC_PACK, s, launch_pack(c, r, coarse ? c->c0 : nullptr, s));
     if (coarse) {
       DD_CUDA(cudaEventRecord(c->ev_fork, s));
       DD_CUDA(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
@@ -345,8 +333,15 @@ void precond(dd_ctx* c, const double* r, int mode, double* zout = nullptr, bool 
     if (rc != DD_OK) throw Error(rc, "local GEMM launch failed");
     if (coarse) DD_CUDA(cudaStreamWaitEvent(s, c->ev_join, 0));
   } else {
-    TIMED(KC_LOCAL_FP64, s, launch_band_solve_local(c, r, c0, s));
-    if (coarse) TIMED(KC_CSOLVE, s, launch_coarse_solve(c, s));
+    if (coarse) {
+      DD_CUDA(cudaEventRecord(c->ev_fork, s));
+      DD_CUDA(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
+      TIMED(KC_CRESTRICT, c->side, launch_coarse_restrict(c, r, c->side));
+      TIMED(KC_CSOLVE, c->side, launch_coarse_solve(c, c->side));
+      DD_CUDA(cudaEventRecord(c->ev_join, c->side));
+    }
+    TIMED(KC_LOCAL_FP64, s, launch_block_solve(c, r, s));
+    if (coarse) DD_CUDA(cudaStreamWaitEvent(s, c->ev_join, 0));
   }
   TIMED(KC_PROLONG, s, launch_prolong(c, mode, s, zout, packed));
 }
@@ -795,7 +790,6 @@ int dd_coarse_build(dd_ctx* c) {
     reset_graph(c);
     int* flag = c->dev_err + 3;
     DD_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), c->stream));
-    const size_t bsz = (size_t)c->ntypes * c->nloc_max * (c->band + 1);
     // the coarse matrix A_0 = Z^T A_sigma Z does not depend on the local factors: it is
     // assembled on the side stream while the local matrices are factored and inverted (those
     // run on a few SMs and leave the GPU mostly idle)
@@ -809,6 +803,7 @@ int dd_coarse_build(dd_ctx* c) {
       // the mixed form only forms A_T^{-1} from the factor and rounds it to BF16/TF32/E4M3:
       // an FP32 factor and FP32 solves are far more accurate than that rounding
       if (!c->bandCB32) {
+        const size_t bsz = (size_t)c->ntypes * c->nloc_max * (c->band + 1);
         c->bandCB32 = (float*)dev_alloc(c, sizeof(float) * bsz);
         c->bandRB32 = (float*)dev_alloc(c, sizeof(float) * bsz);
         c->bandInv32 = (float*)dev_alloc(c, sizeof(float) * (size_t)c->ntypes * c->nloc_max);
@@ -817,13 +812,7 @@ int dd_coarse_build(dd_ctx* c) {
       launch_band_factor(c, c->bandCB32, c->bandRB32, c->bandInv32, c->ntypes, c->nloc_max, c->band, flag,
                          c->type_nloc);
     } else {
-      if (!c->bandCB) {
-        c->bandCB = (double*)dev_alloc(c, sizeof(double) * bsz);
-        c->bandRB = (double*)dev_alloc(c, sizeof(double) * bsz);
-        c->bandInv = (double*)dev_alloc(c, sizeof(double) * (size_t)c->ntypes * c->nloc_max);
-      }
-      launch_local_assemble(c, c->bandCB);
-      launch_band_factor(c, c->bandCB, c->bandRB, c->bandInv, c->ntypes, c->nloc_max, c->band, flag, c->type_nloc);
+      block_factor(c, flag);
     }
     int fl = 0;
     DD_CUDA(cudaMemcpyAsync(&fl, flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
@@ -1412,10 +1401,8 @@ int dd_set_option(dd_ctx* c, int option, int value) {
     case DD_OPT_LOCAL_RHS: {
       if (value != 0 && value != 1 && value != 2 && value != 4)
         return fail(c, DD_EINVAL, "local right-hand sides per warp must be 0, 1, 2 or 4");
-      const int kmax = rhs_per_warp(c->nloc_max, c->band);
-      const int k = value == 0 ? std::min(2, kmax) : std::min(value, kmax);
       try {
-        set_local_groups(c, k);
+        if (c->grid.precision == DD_PREC_FP64) block_groups(c, value);
       } catch (const Error& e) {
         return fail(c, e.code, e.msg);
       }

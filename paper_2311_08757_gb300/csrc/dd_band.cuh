@@ -249,21 +249,4 @@ inline size_t band_ring_bytes(int b, size_t es = sizeof(double)) {
   return r;
 }
 
-// largest number of right-hand sides per warp for local vectors of n_max doubles (shared
-// memory per warp); the local solves use two where allowed (measured fastest at h = 1/32)
-inline int rhs_per_warp(int nmax, int b) {
-  if (b > 128) return 1;   // wide bands: one vector per warp (registers)
-  const size_t per = (size_t)nmax * sizeof(double);
-  if (4 * per <= 48 * 1024) return 4;
-  if (2 * per <= 64 * 1024) return 2;
-  return 1;
-}
-
-#define DD_K_DISPATCH(k, BODY)                              \
-  do {                                                      \
-    if ((k) == 4) { constexpr int KR = 4; BODY; }           \
-    else if ((k) == 2) { constexpr int KR = 2; BODY; }      \
-    else { constexpr int KR = 1; BODY; }                    \
-  } while (0)
-
 }  // namespace dd

@@ -189,9 +189,11 @@ struct dd_ctx {
   int4* subrow = nullptr;           // device, per subdomain: {row offset in Y (slot kpad), type kpad, w2, nloc}
   int* slot_of_sub = nullptr;       // device: subdomain id -> packed row (type-sorted)
   int* sub_of_slot = nullptr;       // device: packed row -> subdomain id
-  int2* groups = nullptr;           // device: {first slot, count} of same-type slots solved by one warp
-  int ngroups = 0, rhs_k = 1;       // FP64 local solves: groups and right-hand sides per warp
-  std::vector<int2> group_h;        // host copy of groups
+  int rep_of_type[dd::kMaxTypes];   // a subdomain of each type
+  // FP64 local solves (k_block.cu): same-type slots solved by one cluster {first slot, count} and
+  // the launch shape (blocks per side, subdomains per block, column ranges, row warps, row groups)
+  int2* groups = nullptr;
+  int ngroups = 0, blk_cr = 1, blk_R = 1, blk_PW = 1, blk_RW = 1, blk_rgl = 1;
   int nloc_max = 0, kpad = 0, band = 0;
 
   // V and stencil tables [tap][cls]
@@ -243,12 +245,10 @@ struct dd_ctx {
   double *stage_a = nullptr, *stage_b = nullptr;         // unpadded staging (ndof)
 
   // local solves
-  double* bandCB = nullptr;   // [type][nloc_max][band+1] column band of L
-  double* bandRB = nullptr;   // [type][nloc_max][band+1] row band of L
-  double* bandInv = nullptr;  // [type][nloc_max] 1/L_ii
-  float* bandCB32 = nullptr;  // the same in FP32: the mixed form, whose inverses are rounded
-  float* bandRB32 = nullptr;
-  float* bandInv32 = nullptr;
+  double* blkS = nullptr;     // FP64: [type][plane] inverse Schur complements of the local matrices
+  float* bandCB32 = nullptr;  // mixed form: [type][nloc_max][band+1] column band of L (its inverse is rounded)
+  float* bandRB32 = nullptr;  // [type][nloc_max][band+1] row band of L
+  float* bandInv32 = nullptr; // [type][nloc_max] 1/L_ii^2
   double* Y64 = nullptr;      // [nsub][kpad] local solutions (FP64 path)
   float* Y32 = nullptr;       // [nsub][kpad] local solutions (GEMM path)
   void* Ainv = nullptr;       // [type][kpad][kpad] rounded local inverses
@@ -376,7 +376,9 @@ void launch_local_assemble(dd_ctx* c, T* CB);
 // banded Cholesky of nmat matrices (orders in sizes_host, or all n when null); T double or float
 template <typename T>
 int launch_band_factor(dd_ctx* c, T* CB, T* RB, T* inv, int nmat, int n, int b, int* flag, const int* sizes_host);
-void launch_band_solve_local(dd_ctx* c, const double* r, double* c0, cudaStream_t s);
+void block_factor(dd_ctx* c, int* flag);           // FP64: inverse Schur complements of every type
+void block_groups(dd_ctx* c, int want);            // launch shape (want: subdomains per block, 0: chosen)
+void launch_block_solve(dd_ctx* c, const double* r, cudaStream_t s);
 template <typename T>
 void launch_band_inverse_rows(int n, int b, const T* CB, const T* RB, const T* inv, T* out, cudaStream_t s);
 

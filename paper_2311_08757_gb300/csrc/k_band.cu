@@ -1,5 +1,4 @@
-// Local subdomain matrices and their banded Cholesky factors; the FP64 local solves of
-// the plain method; the cell eigenpair.
+// Local subdomain matrices and their banded Cholesky factors (mixed form); the cell eigenpair.
 //
 // Local problems (Sec. 3.1): A_{sigma,i} = R_i A_sigma R_i^T on the interior nodes strictly
 // inside the open overlapping box Omega_i (homogeneous Dirichlet on its artificial
@@ -391,90 +390,7 @@ void launch_local_assemble(dd_ctx* c, T* CB) {
   DD_CUDA(cudaGetLastError());
   DD_CUDA(cudaFreeAsync(drep, c->stream));
 }
-template void launch_local_assemble<double>(dd_ctx*, double*);
 template void launch_local_assemble<float>(dd_ctx*, float*);
-
-// ----------------------------------------------------------------------------------------
-// FP64 local solves y_i = A_{sigma,i}^{-1} R_i r for every subdomain (one warp each); the
-// result goes to Y[slot(i)][k]; the prolong-sum gathers it.
-// ----------------------------------------------------------------------------------------
-template <int NV, int PF, int K>
-__global__ void k_local_solve(Geo g, const Sub* __restrict__ subs, const int2* __restrict__ groups, int ngroups,
-                              const int* __restrict__ sub_of_slot, const double* __restrict__ r,
-                              const double* __restrict__ CB, const double* __restrict__ RB,
-                              const double* __restrict__ inv, int nmax, int b, double* __restrict__ Y, int kpad,
-                              const double* __restrict__ wT, double* c0, const PcgState* st) {
-  if (st != nullptr && st->done) return;
-  extern __shared__ double xs_all[];
-  const int wpb = blockDim.x >> 5;
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int gi = blockIdx.x * wpb + wid;
-  if (gi >= ngroups) return;
-  const int2 grp = groups[gi];   // K (or fewer) consecutive slots of one type
-  constexpr int RING = band_ring_elems<NV, PF>();
-  double* xs = xs_all + (size_t)wid * (K * nmax + RING);
-  double* ring = xs + (size_t)K * nmax;
-  const int type = subs[sub_of_slot[grp.x]].type;
-  int n = 0;
-#pragma unroll
-  for (int j = 0; j < K; ++j) {
-    double* xj = xs + (size_t)j * nmax;
-    if (j < grp.y) {
-      const int s = sub_of_slot[grp.x + j];
-      const Sub sb = subs[s];
-      n = sb.nloc;
-      // gather R_i r; the coarse right-hand side (D_i R_i psi)^T r rides along (Def. 2.1)
-      double cr = 0.0;
-      const double* wt = wT + (size_t)type * kpad;
-      for (int k = lane; k < sb.nloc; k += 32) {
-        const int sj = k % g.nyi, cc = k / g.nyi;
-        const int c1 = cc / sb.w2, c2 = cc % sb.w2;
-        long long idx;
-        if (g.p == 1) idx = (long long)(sb.lo1 + c1) * g.Ypad + sj;
-        else idx = ((long long)(sb.lo1 + c1) * g.ncx + (sb.lo2 + c2)) * g.Ypad + sj;
-        const double v = r[idx];
-        xj[k] = v;
-        if (c0 != nullptr) cr = fma(wt[loc_pad(g, k)], v, cr);
-      }
-      if (c0 != nullptr) {
-        cr = warp_sum(cr);
-        if (lane == 0) c0[s] = cr;
-      }
-    } else {
-      for (int k = lane; k < nmax; k += 32) xj[k] = 0.0;
-    }
-  }
-  const size_t off = (size_t)type * nmax;
-  band_solve_k<NV, PF, K>(xs, nmax, n, b, CB + off * (b + 1), RB + off * (b + 1), inv + off, ring);
-  __syncwarp();
-  for (int j = 0; j < grp.y; ++j) {
-    double* y = Y + (size_t)(grp.x + j) * kpad;
-    for (int k = lane; k < n; k += 32) y[loc_pad(g, k)] = xs[(size_t)j * nmax + k];
-  }
-}
-
-void launch_band_solve_local(dd_ctx* c, const double* r, double* c0, cudaStream_t s) {
-  const int K = c->rhs_k;
-  const int wpb = 1;
-  const size_t smem = sizeof(double) * (size_t)K * c->nloc_max + band_ring_bytes(c->band);
-  const int nb = c->ngroups;
-  DD_BAND_DISPATCH(c->band, {
-    DD_K_DISPATCH(K, {
-      constexpr int KK = (NV == 0 || NV > 4) ? 1 : KR;
-      if (K > KK) throw Error(DD_EINVAL, "local right-hand sides per warp exceed the kernel's");
-      static PerDeviceOnce attr_set;   // once per device and instance
-      once_per_device(attr_set, [] {
-        DD_CUDA(cudaFuncSetAttribute(k_local_solve<NV, PF, KK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     220 * 1024));
-      });
-      (k_local_solve<NV, PF, KK><<<nb, wpb * 32, smem, s>>>(c->g, c->subs, c->groups, c->ngroups, c->sub_of_slot,
-                                                           r, c->bandCB, c->bandRB, c->bandInv, c->nloc_max,
-                                                           c->band, c->Y64, c->kpad, c->wT, c0, c->st),
-       dd::note_launch());
-    });
-  });
-  DD_CUDA(cudaGetLastError());
-}
 
 // ----------------------------------------------------------------------------------------
 // Cell eigenpair (cell problem of Sec. 1 / weak cell problem of Sec. 2): lowest eigenpair of
