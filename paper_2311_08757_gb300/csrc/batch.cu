@@ -45,8 +45,8 @@ struct BGroup {
   std::vector<BInst> Bh;
   BInst* B = nullptr;
   int2 *vm_init = nullptr, *vm_fused = nullptr, *vm_xr = nullptr, *vm_prolong = nullptr, *vm_sdot = nullptr,
-       *vm_st = nullptr, *vm_st2 = nullptr, *vm_vec = nullptr, *vm_pack = nullptr;
-  int n_init = 0, n_fused = 0, n_xr = 0, n_prolong = 0, n_sdot = 0, n_st = 0, n_st2 = 0, n_vec = 0, n_pack = 0;
+       *vm_st = nullptr, *vm_st2 = nullptr, *vm_vec = nullptr, *vm_pack = nullptr, *vm_lop = nullptr;
+  int n_init = 0, n_fused = 0, n_xr = 0, n_prolong = 0, n_sdot = 0, n_st = 0, n_st2 = 0, n_vec = 0, n_pack = 0, n_lop = 0;
   size_t cr_smem = 0;
   int ypad = 0, precision = 0, check_every = 8;
   bool arith = true;               // every instance's prolong-sum owners in closed form
@@ -99,7 +99,7 @@ void free_group(BGroup* g) {
   if (g->graph) cudaGraphExecDestroy(g->graph);
   dd::bgemm_destroy(g->gemm);
   for (void* p : {(void*)g->B, (void*)g->vm_init, (void*)g->vm_fused, (void*)g->vm_xr, (void*)g->vm_prolong,
-                  (void*)g->vm_sdot, (void*)g->vm_st, (void*)g->vm_st2, (void*)g->vm_vec, (void*)g->vm_pack,
+                  (void*)g->vm_sdot, (void*)g->vm_st, (void*)g->vm_st2, (void*)g->vm_vec, (void*)g->vm_pack, (void*)g->vm_lop,
                   (void*)g->stat_d, (void*)g->xptr_d, (void*)g->err_d})
     if (p) cudaFree(p);
   if (g->stat_h) cudaFreeHost(g->stat_h);
@@ -244,7 +244,7 @@ BGroup* build_group(dd_batch* b, const std::vector<int>& idx) {
     DD_CUDA(cudaMalloc(&g->err_d, sizeof(int) * 16));
     DD_CUDA(cudaMemset(g->err_d, 0, sizeof(int) * 16));
     g->Bh.assign(n, BInst());
-    std::vector<int2> vinit, vfused, vxr, vprol, vsdot, vst, vst2, vvec, vpack;
+    std::vector<int2> vinit, vfused, vxr, vprol, vsdot, vst, vst2, vvec, vpack, vlop;
     std::vector<dd_ctx*> cs;
     std::vector<int> tb, sb;
     std::vector<double*> xs;
@@ -291,6 +291,7 @@ BGroup* build_group(dd_batch* b, const std::vector<int>& idx) {
       for (int k = 0; k < I.nb_st; ++k) vst.push_back(make_int2(j, k));
       for (int k = 0; k < I.nb_st2; ++k) vst2.push_back(make_int2(j, k));
       for (int k = 0; k < I.nb_vec; ++k) vvec.push_back(make_int2(j, k));
+      for (int k = 0; k < I.nb_lop; ++k) vlop.push_back(make_int2(j, k));
       for (int k = 0; k < c->g.nsub; ++k) vpack.push_back(make_int2(j, k));
     }
     if (g->cr_smem > 220 * 1024) throw dd::Error(DD_EINVAL, "coarse chain too long for the batched cyclic reduction");
@@ -303,6 +304,7 @@ BGroup* build_group(dd_batch* b, const std::vector<int>& idx) {
     g->vm_st = upload_vmap(vst); g->n_st = (int)vst.size();
     g->vm_st2 = upload_vmap(vst2); g->n_st2 = (int)vst2.size();
     g->vm_vec = upload_vmap(vvec); g->n_vec = (int)vvec.size();
+    g->vm_lop = upload_vmap(vlop); g->n_lop = (int)vlop.size();
     g->vm_pack = upload_vmap(vpack); g->n_pack = (int)vpack.size();
     DD_CUDA(cudaMalloc(&g->B, sizeof(BInst) * n));
     DD_CUDA(cudaMemcpy(g->B, g->Bh.data(), sizeof(BInst) * n, cudaMemcpyHostToDevice));
@@ -639,7 +641,7 @@ int run_lopcg_fused(dd_batch* b, BGroup* g, const Ready& ready, const Outputs& o
     launch_b_stencil2(g->B, g->vm_st2, g->n_st2, BV_Z, R(AW), R(MW), s);
     const int S[3] = {R(X), BV_Z, R(XP)}, AS[3] = {R(AX), R(AW), R(AXP)}, MS[3] = {R(MX), R(MW), R(MXP)};
     launch_b_lop_gram(g->B, g->vm_vec, g->n_vec, S, AS, MS, 1e-10, s);
-    launch_b_lop_update3(g->B, g->vm_vec, g->n_vec, S, AS, MS, R(T), R(AT), R(MT), R(RO), s);
+    launch_b_lop_update3(g->B, g->vm_lop, g->n_lop, S, AS, MS, R(T), R(AT), R(MT), R(RO), s);
     int t0 = XP;
     XP = X; X = T; T = t0;
     t0 = AXP; AXP = AX; AX = AT; AT = t0;

@@ -51,6 +51,37 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
       return;
     }
   }
+  if constexpr (NV > 4) {
+    if (blockDim.x <= 256 && (blockDim.x & 31) == 0) {
+      // The additions of the shuffle tree below, in the same order, from shared memory: a level
+      // with o sums per warp and value is packed into full warps, so the FP64 pipe, which
+      // charges a warp instruction whatever its active lanes, sees 31 / 32 of an instruction per
+      // warp and value instead of 5 (15 values, 8 warps: 116 + 105 against 675).
+      __shared__ double st[NV][256];
+#pragma unroll
+      for (int k = 0; k < NV; ++k) st[k][threadIdx.x] = v[k];
+      __syncthreads();
+#pragma unroll
+      for (int lo = 4; lo >= 0; --lo) {
+        const int o = 1 << lo;
+        for (int e = threadIdx.x; e < (NV * nw) << lo; e += blockDim.x) {
+          const int i = e & (o - 1), kw = e >> lo, k = kw / nw, w = kw - k * nw;
+          st[k][w * 32 + i] += st[k][w * 32 + i + o];
+        }
+        __syncthreads();
+      }
+      if (threadIdx.x < NV) {   // the warps' sums, as one more shuffle tree would add them
+        double* t = st[threadIdx.x];
+        for (int o = 16; o > 0; o >>= 1)
+          for (int i = 0; i < o && i + o < nw; ++i) t[32 * i] += t[32 * (i + o)];
+      }
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < NV; ++k) v[k] = st[k][0];
+      __syncthreads();
+      return;
+    }
+  }
   __shared__ double sm[32][NV];
 #pragma unroll
   for (int k = 0; k < NV; ++k) v[k] = warp_sum(v[k]);

@@ -323,7 +323,7 @@ struct BInst {
   const double* cr;       // cyclic-reduction coefficients of A_0 (p = 1)
   int cr_m, cr_c2, cr_w2, cr_staged;
   int kpad, coarse, nsub, flexible;
-  int nb_init, nb_fused, nb_xr, nb_prolong, nb_sdot, nb_st, nb_vec, nb_st2;
+  int nb_init, nb_fused, nb_xr, nb_prolong, nb_sdot, nb_st, nb_vec, nb_st2, nb_lop;
   int active;             // 0 once the problem's eigen-iteration has stopped
   int* err;               // the context's error word of bounded waits
   double* lop[12];        // SI-LOPCG work vectors (padded)
@@ -347,6 +347,7 @@ struct BStat {
 
 // ----- launchers (kernels in k_*.cu) -----
 int grid_blocks(long long work, int threads, int max_per_sm = 8);
+int lop_blocks(long long n);   // SI-LOPCG update pass over n entries
 
 void launch_build_tables(dd_ctx* c);
 void launch_tabS(dd_ctx* c, double sigma);

@@ -9,6 +9,11 @@ namespace dd {
 
 // Gram matrices (upper triangles) of S = [x, w, xp] under A_sigma and M, and the sums of the
 // three vectors; then the Rayleigh-Ritz step in the last block.
+//
+// Bound by the FP64 pipe: 15 multiply-adds per entry, 50 us at 2.1M entries, against 22 us for
+// the nine vectors at the copy rate; the block sums of 15 values come on top (block_sum).  The
+// iteration amplifies the rounding of these sums (x_k and x_{k-1} are nearly parallel), so their
+// order is fixed: entries grid-stride over grid_blocks(n) blocks, then the shuffle tree.
 __device__ __forceinline__ void lop_gram_body(VBlk vb, long long n, const double* __restrict__ x,
                                                        const double* __restrict__ w, const double* __restrict__ xp,
                                                        const double* __restrict__ Ax, const double* __restrict__ Aw,
@@ -19,6 +24,7 @@ __device__ __forceinline__ void lop_gram_body(VBlk vb, long long n, const double
   double acc[15];
 #pragma unroll
   for (int k = 0; k < 15; ++k) acc[k] = 0.0;
+#pragma unroll 2
   for (long long t = (long long)vb.b * blockDim.x + threadIdx.x; t < n;
        t += (long long)vb.nb * blockDim.x) {
     const double s0 = x[t], s1 = w[t], s2 = xp[t];
@@ -81,6 +87,10 @@ __global__ void __launch_bounds__(kThreads) k_lop_update(long long n, const doub
     out[t] = fma(c2, xp[t], fma(c1, w[t], c0 * x[t]));
 }
 
+// blocks of the update pass: two per SM, two entries per thread and step.  It reads and writes 13
+// vectors (32 us at the copy rate for 2.1M entries) and needs 13 FP64 instructions per entry (43 us)
+int lop_blocks(long long n) { return grid_blocks(n / 2, kThreads, 2); }
+
 // x_{k+1} = S c together with its images A_sigma x_{k+1} = (A_sigma S) c and M x_{k+1} = (M S) c
 // (linear combinations instead of two more stencil passes), the outer residual
 // r_o = A_sigma x - theta M x and the norms of the stop test.  c is M-normalised by the
@@ -95,19 +105,27 @@ __device__ __forceinline__ void lop_update3_body(VBlk vb, long long n, const dou
                                                           double* partials, unsigned* counter) {
   const double c0 = ls->c[0], c1 = ls->c[1], c2 = ls->c[2], th = ls->theta;
   double acc[3] = {0.0, 0.0, 0.0};
-  for (long long t = (long long)vb.b * blockDim.x + threadIdx.x; t < n;
+  auto ld = [](const double* p, long long t) { return reinterpret_cast<const double2*>(p)[t]; };
+  auto st = [](double* p, long long t, double2 v) { reinterpret_cast<double2*>(p)[t] = v; };
+  auto comb = [&](double u, double v, double w) { return fma(c2, w, fma(c1, v, c0 * u)); };
+  for (long long t = (long long)vb.b * blockDim.x + threadIdx.x; t < n / 2;
        t += (long long)vb.nb * blockDim.x) {
-    const double xv = fma(c2, s2[t], fma(c1, s1[t], c0 * s0[t]));
-    const double av = fma(c2, a2[t], fma(c1, a1[t], c0 * a0[t]));
-    const double mv = fma(c2, m2[t], fma(c1, m1[t], c0 * m0[t]));
-    const double e = fma(-th, mv, av);
-    x[t] = xv;
-    ax[t] = av;
-    mx[t] = mv;
-    ro[t] = e;
-    acc[0] = fma(e, e, acc[0]);
-    acc[1] = fma(mv, mv, acc[1]);
-    acc[2] = fma(xv, mv, acc[2]);
+    const double2 u0 = ld(s0, t), u1 = ld(s1, t), u2 = ld(s2, t), b0 = ld(a0, t), b1 = ld(a1, t), b2 = ld(a2, t);
+    const double2 d0 = ld(m0, t), d1 = ld(m1, t), d2 = ld(m2, t);
+    const double2 xv = make_double2(comb(u0.x, u1.x, u2.x), comb(u0.y, u1.y, u2.y));
+    const double2 av = make_double2(comb(b0.x, b1.x, b2.x), comb(b0.y, b1.y, b2.y));
+    const double2 mv = make_double2(comb(d0.x, d1.x, d2.x), comb(d0.y, d1.y, d2.y));
+    const double2 e = make_double2(fma(-th, mv.x, av.x), fma(-th, mv.y, av.y));
+    st(x, t, xv);
+    st(ax, t, av);
+    st(mx, t, mv);
+    st(ro, t, e);
+    acc[0] = fma(e.x, e.x, acc[0]);
+    acc[1] = fma(mv.x, mv.x, acc[1]);
+    acc[2] = fma(xv.x, mv.x, acc[2]);
+    acc[0] = fma(e.y, e.y, acc[0]);
+    acc[1] = fma(mv.y, mv.y, acc[1]);
+    acc[2] = fma(xv.y, mv.y, acc[2]);
   }
   double tot[3];
   if (grid_sum_last<3>(acc, partials, counter, tot, vb) && threadIdx.x == 0) {
@@ -174,7 +192,7 @@ __global__ void __launch_bounds__(kThreads, 4) kb_lop_update3(const BInst* __res
   const int2 m = vmap[blockIdx.x];
   const BInst& I = B[m.x];
   if (!I.active) return;
-  lop_update3_body(VBlk{m.y, I.nb_vec}, I.g.plen, lvec(I, R.s[0]), lvec(I, R.s[1]), lvec(I, R.s[2]),
+  lop_update3_body(VBlk{m.y, I.nb_lop}, I.g.plen, lvec(I, R.s[0]), lvec(I, R.s[1]), lvec(I, R.s[2]),
                    lvec(I, R.a[0]), lvec(I, R.a[1]), lvec(I, R.a[2]), lvec(I, R.m[0]), lvec(I, R.m[1]),
                    lvec(I, R.m[2]), lvec(I, x_role), lvec(I, ax_role), lvec(I, mx_role), lvec(I, ro_role), I.lst,
                    I.lop_red, I.cnt + CNT_LOP);
@@ -234,8 +252,7 @@ void launch_b_lop_reset(const BInst* B, int n, cudaStream_t s) {
 void launch_lop_gram(dd_ctx* c, const double* const S[3], const double* const AS[3], const double* const MS[3],
                      double drop, cudaStream_t s) {
   const long long n = c->g.plen;
-  const int nb = grid_blocks(n, kThreads);
-  (k_lop_gram<<<nb, kThreads, 0, s>>>(n, S[0], S[1], S[2], AS[0], AS[1], AS[2], MS[0], MS[1], MS[2], c->lst,
+  (k_lop_gram<<<grid_blocks(n, kThreads), kThreads, 0, s>>>(n, S[0], S[1], S[2], AS[0], AS[1], AS[2], MS[0], MS[1], MS[2], c->lst,
                                        c->lop_red, c->cnt + CNT_LOP, drop),
    dd::note_launch());
   DD_CUDA(cudaGetLastError());
@@ -251,7 +268,7 @@ void launch_lop_update(dd_ctx* c, const double* x, const double* w, const double
 void launch_lop_update3(dd_ctx* c, const double* const S[3], const double* const AS[3], const double* const MS[3],
                         double* x, double* Ax, double* Mx, double* ro, cudaStream_t s) {
   const long long n = c->g.plen;
-  (k_lop_update3<<<grid_blocks(n, kThreads), kThreads, 0, s>>>(n, S[0], S[1], S[2], AS[0], AS[1], AS[2], MS[0], MS[1],
+  (k_lop_update3<<<lop_blocks(n), kThreads, 0, s>>>(n, S[0], S[1], S[2], AS[0], AS[1], AS[2], MS[0], MS[1],
                                                                 MS[2], x, Ax, Mx, ro, c->lst, c->lop_red,
                                                                 c->cnt + CNT_LOP),
    dd::note_launch());

@@ -1767,6 +1767,7 @@ void batch_grid_sizes(const dd_ctx* c, BInst* I) {
   I->nb_st = resident_grid(k_stencil<1, false>, w, kThreads);
   I->nb_vec = grid_blocks(g.plen, kThreads);
   I->nb_st2 = resident_grid(k_stencil2<1>, w, kThreads);
+  I->nb_lop = lop_blocks(g.plen);
 }
 
 void launch_b_zero_roles(const BInst* B, const int2* vmap, int nvb, int first_role, int nroles, cudaStream_t s) {
