@@ -167,7 +167,7 @@ struct dd_ctx {
   int4 ptypes = {0, 0, 0, 0};       // p = 1: type ids of the left end, interior and right end subdomains
   int pdl = 0;                      // PCG chain kernels launched with programmatic dependent launch
   int fuse_xr_opt = 0;              // x/r update fused into the packing: 1 on, 0 or -1 off
-  int matvec_tiled = 1;             // p = 2 float pairs: the shared-memory tiled matvec where it fits
+  int matvec_tiled = 1;             // p = 2 float pairs: the register-table matvec where it fits
   // x_{k+1} = x_k + alpha_k p_k deferred to iteration k + 1's p update, which reads p_k anyway,
   // and one final update after the last iteration: the x/r update then streams r and q only
   int x_lag = 1;

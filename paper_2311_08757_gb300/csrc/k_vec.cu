@@ -10,7 +10,7 @@
 #include <map>
 #include <mutex>
 
-#include "dd_common.cuh"
+#include "dd_async.cuh"
 
 namespace dd {
 
@@ -853,85 +853,176 @@ __global__ void __launch_bounds__(kThreads) k_matvec_pq_pairs(Geo g, const float
   }
 }
 
-// The same pass tiled through shared memory.  The class of node (a1, a2, slot) is
-// ((a1 mod n) n + a2 mod n) Ypad + slot, so a block that takes only planes a1 = r (mod n)
-// needs n Ypad classes of the table: it stages that slice once (n Ypad rows of 28 float
-// pairs), then walks its share of the residue's (plane, a2 tile) pairs; each tile (one plane,
-// TA = blockDim / Ypad node columns, one node per thread) stages the split p of the planes
-// a1 - 1 .. a1 + 1 over columns a2 - 1 .. a2 + TA, so every tap reads shared memory.  Each
-// node's arithmetic is that of k_matvec_pq_pairs (the same q bits); the (p, q) partials are
-// summed in another order.
-constexpr int kTiledMaxClasses = 448;   // n Ypad <= 448: the table slice is at most 98 KB
+// The same pass with the table in registers.  The class of node (a1, a2, slot) depends on a1 and
+// a2 modulo n, so a block takes the planes of one residue r = a1 mod n and, of every cell along x_2,
+// the same W columns: a thread then holds one class for the whole kernel, and its 27 split taps
+// stay in registers.  Per step the block evaluates
+// kClsCells cells of one plane, and every operation of pair_fma works on two of the thread's nodes
+// at once (packed FP32 instructions; the packed two-product negates one factor beforehand, an exact
+// operation).  The split p of the planes a1 - 1 .. a1 + 1 over W + 2 columns is one contiguous run per
+// plane and cell, brought by bulk copies two steps ahead.  Each node's arithmetic is that of k_matvec_pq_pairs, operation by
+// operation (the same q bits); the (p, q) partials are summed in another order.
+//
+// L = 64, h = 1/16 (17M padded nodes): 525-590 us with the table slice and p staged through shared
+// memory by the threads (one cell, scalar operations), 375 us with two cells of 256 threads, 345 us
+// with four cells of 128 threads; the FP32 pipe needs 146 us for its 27 x 13 packed operations per
+// two nodes, the copies 134 + 3.4 x 134 MB mostly from L2.  What is left is the moves that pair the
+// operands and the 12 warps an SM holds at 122 registers.
+constexpr int kClsThreads = 128;
 
-__global__ void __launch_bounds__(kThreads) k_matvec_pq_pairs_tiled(Geo g, const float2* __restrict__ tab2,
-                                                                    const float2* __restrict__ p2, double* pb0,
-                                                                    double* pb1, double* __restrict__ q,
-                                                                    PcgState* st, double* partials,
-                                                                    unsigned* counter) {
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+
+// pair_fma for two nodes with the same coefficient, t = (th, th), tm = (tl, tl): the same roundings,
+// with the product and its negative exchanged where that saves a negation
+__device__ __forceinline__ void pair_fma2(f32x2 t, f32x2 tm, f32x2 xh, f32x2 xl, f32x2& s, f32x2& c) {
+  const f32x2 np = mul2(t, mul2(xh, pack2(-1.0f, -1.0f)));   // -p
+  const f32x2 e = fma2(t, xh, np);                      // th * xh = p + e exactly
+  const f32x2 u = sub2(s, np);                          // s + p
+  const f32x2 bv = sub2(u, s);
+  const f32x2 err = sub2(sub2(s, sub2(u, bv)), add2(np, bv));   // s + p = u + err
+  s = u;
+  c = add2(c, add2(e, err));
+  c = fma2(t, xl, c);
+  c = fma2(tm, xh, c);
+}
+
+constexpr int kClsStages = 3, kClsCells = 4;
+constexpr int ERR_MATVEC_WAIT = 1 << 9;   // error-word bit: a tile of the matvec did not arrive in time
+// float2 elements of one cell's staged planes, with two zero elements on each side
+__host__ __device__ inline int cls_cell_len(int CW, int Y) { return 3 * (CW + 2) * Y + 4; }
+
+__global__ void __launch_bounds__(kClsThreads, 3) k_matvec_pq_pairs_cls(Geo g, const float2* __restrict__ tab2,
+                                                                        const float2* __restrict__ p2, double* pb0,
+                                                                        double* pb1, double* __restrict__ q,
+                                                                        PcgState* st, double* partials,
+                                                                        unsigned* counter, int CW, int ncg, int* err) {
   pdl_enter();
   if (st->done) return;
-  extern __shared__ __align__(16) float4 smt[];
+  extern __shared__ __align__(16) float2 smt[];
+  __shared__ __align__(8) unsigned long long s_bar[kClsStages];
   const int Y = g.Ypad, yl = g.ylog, n = g.n;
-  const int ncls_r = n * Y;                      // classes of one residue
-  const int TA = (int)blockDim.x >> yl;          // node columns per tile (blockDim multiple of Y)
-  float2* tabs = reinterpret_cast<float2*>(smt);                    // [ncls_r][28]
-  float2* tile_raw = tabs + (size_t)ncls_r * kPairTapStride3;       // guard, [3][TA + 2][Y], guard
-  float2* tile = tile_raw + 1;
-  const int row = (TA + 2) * Y;                  // one plane's staged run
-  const int nbr = (int)gridDim.x / n;            // blocks per residue
-  const int r = (int)blockIdx.x % n, kb = (int)blockIdx.x / n;
-  // the residue's table slice: classes (r n + m) Y + slot for m < n
-  {
-    const float4* src = reinterpret_cast<const float4*>(tab2 + (size_t)r * ncls_r * kPairTapStride3);
-    float4* dst = smt;
-    for (int e = threadIdx.x; e < ncls_r * (kPairTapStride3 / 2); e += blockDim.x) dst[e] = __ldg(src + e);
-  }
-  if (threadIdx.x == 0) {
-    tile_raw[0] = make_float2(0.0f, 0.0f);
-    tile_raw[3 * row + 1] = make_float2(0.0f, 0.0f);
-  }
-  const double* __restrict__ p = p_cur(pb0, pb1, st->iter);
+  const int ngrp = n * ncg, gid = (int)blockIdx.x % ngrp, kb = (int)blockIdx.x / ngrp, nbr = (int)gridDim.x / ngrp;
+  const int r = gid / ncg, c0 = (gid % ncg) * CW, W = min(CW, n - c0);
+  const int row = (W + 2) << yl;                 // one plane's staged run
+  const int cell = cls_cell_len(CW, Y);          // a stage holds kClsCells of them
+  const int cl = (int)threadIdx.x >> yl, slot = (int)threadIdx.x & (Y - 1);
+  const bool mine = cl < W;
   const int a1_first = (r == 0) ? n : r;
   const int nplanes = (a1_first <= g.nxi) ? (g.nxi - a1_first) / n + 1 : 0;
-  const int ntile2 = (g.nxi + TA - 1) / TA;
-  const long long ntiles = (long long)nplanes * ntile2;
-  const long long c1 = (long long)g.ncx * Y;
-  const int c = (int)threadIdx.x >> yl, slot = (int)threadIdx.x & (Y - 1);
-  double acc[1] = {0.0};
-  for (long long tt = kb; tt < ntiles; tt += nbr) {
-    const int a1 = a1_first + n * (int)(tt / ntile2);
-    const int a2_0 = 1 + TA * (int)(tt % ntile2);
-    __syncthreads();   // the previous tile's taps are read (and, the first time, the table staged)
-    for (int e = threadIdx.x; e < 3 * row; e += blockDim.x) {
-      const int pl = e / row, w = e - pl * row;
-      const int col = a2_0 - 1 + (w >> yl);
-      tile[e] = (col <= g.nxi + 1) ? p2[(long long)(a1 - 1 + pl) * c1 + (long long)col * Y + (w & (Y - 1))]
-                                   : make_float2(0.0f, 0.0f);
+  const int nset = (g.L + kClsCells - 1) / kClsCells;   // sets of kClsCells cells along x_2
+  const int nitem = nplanes * nset;
+  const long long c1 = (long long)g.ncx << yl;
+  const uint32_t bar = smem_u32(s_bar);
+  auto fetch = [&](int it, int sl) {             // by one thread: the planes of item it into stage sl
+    const int a1 = a1_first + n * (it / nset), j0 = kClsCells * (it % nset), nc = min(kClsCells, g.L - j0);
+    const uint32_t bytes = (uint32_t)row * sizeof(float2);
+    mbar_expect_tx(bar + 8 * sl, 3 * nc * bytes);
+    for (int cb = 0; cb < nc; ++cb)
+      for (int pl = 0; pl < 3; ++pl)
+        bulk_g2s(smem_u32(smt + (size_t)(kClsCells * sl + cb) * cell + 2 + pl * row),
+                 p2 + (long long)(a1 - 1 + pl) * c1 + ((long long)(n * (j0 + cb) + c0 - 1) << yl), bytes, bar + 8 * sl);
+  };
+  for (int e = threadIdx.x; e < 4 * kClsCells * kClsStages; e += blockDim.x) {   // the zero elements around each cell
+    const int k = e & 3;
+    smt[(size_t)(e >> 2) * cell + (k < 2 ? k : 3 * row + k)] = make_float2(0.0f, 0.0f);
+  }
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kClsStages; ++i) mbar_init(bar + 8 * i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    for (int i = 0; i < kClsStages - 1; ++i)
+      if (kb + i * nbr < nitem) fetch(kb + i * nbr, i);
+  }
+  f32x2 th[27], tl[27];
+  {
+    const float4* tr = reinterpret_cast<const float4*>(tab2 + (size_t)((r * n + c0 + (mine ? cl : 0)) * Y + slot) * kPairTapStride3);
+#pragma unroll
+    for (int k4 = 0; k4 < kPairTapStride3 / 2; ++k4) {
+      const float4 tv = __ldg(tr + k4);
+      th[2 * k4] = pack2(tv.x, tv.x);
+      tl[2 * k4] = pack2(tv.y, tv.y);
+      if (2 * k4 + 1 < 27) {
+        th[2 * k4 + 1] = pack2(tv.z, tv.z);
+        tl[2 * k4 + 1] = pack2(tv.w, tv.w);
+      }
     }
-    __syncthreads();
-    const int a2 = a2_0 + c;
-    if (a2 <= g.nxi) {
-      const float4* tr = reinterpret_cast<const float4*>(tabs + (size_t)((a2 % n) * Y + slot) * kPairTapStride3);
-      const float2* x = tile + row + (c + 1) * Y + slot;   // plane a1, column a2 (the centre of the taps)
-      float hs = 0.0f, ls = 0.0f;
+  }
+  const double* __restrict__ p = p_cur(pb0, pb1, st->iter);
+  double acc[1] = {0.0};
+  int sl = 0, ph = 0;
+  bool dead = false;   // a wait gave up: the error word tells the host
+  __syncthreads();
+  for (int it = kb; it < nitem; it += nbr) {
+    // the stage read two steps ago is free: every thread has passed the barrier that ended that step
+    if (threadIdx.x == 0 && it + (kClsStages - 1) * nbr < nitem)
+      fetch(it + (kClsStages - 1) * nbr, sl == 0 ? kClsStages - 1 : sl - 1);
+    if (!dead && !mbar_wait(bar + 8 * sl, (uint32_t)ph, err, ERR_MATVEC_WAIT)) dead = true;
+    if (mine) {
+      const int a1 = a1_first + n * (it / nset), col = kClsCells * n * (it % nset) + c0 + cl;   // in the first cell
+      const long long idx = (long long)a1 * c1 + ((long long)col << yl) + slot, step = (long long)n << yl;
+      bool ok[kClsCells];
+      double pv[kClsCells];
 #pragma unroll
-      for (int k4 = 0; k4 < kPairTapStride3 / 2; ++k4) {
-        const float4 tv = tr[k4];
+      for (int b = 0; b < kClsCells; ++b) {
+        ok[b] = col + b * n >= 1 && col + b * n <= g.nxi;
+        pv[b] = ok[b] ? p[idx + b * step] : 0.0;
+      }
+      const float2* x = smt + (size_t)(kClsCells * sl) * cell + 2 + row + ((cl + 1) << yl) + slot;   // plane a1, this column
+      f32x2 hs[kClsCells / 2], ls[kClsCells / 2];
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int tap = 2 * k4 + j;
-          if (tap < 27) {
-            const int d1 = tap / 9 - 1, d2 = (tap / 3) % 3 - 1, dy = tap % 3 - 1;
-            const float2 xv = x[d1 * row + d2 * Y + dy];
-            pair_fma(j ? tv.z : tv.x, j ? tv.w : tv.y, xv.x, xv.y, hs, ls);
-          }
+      for (int b = 0; b < kClsCells / 2; ++b) hs[b] = ls[b] = 0;
+#pragma unroll
+      for (int tap = 0; tap < 27; ++tap) {
+        const float2* xt = x + (tap / 9 - 1) * row + ((tap / 3) % 3 - 1) * Y + tap % 3 - 1;
+#pragma unroll
+        for (int b = 0; b < kClsCells / 2; ++b) {
+          const float2 va = xt[2 * b * cell], vb = xt[(2 * b + 1) * cell];
+          pair_fma2(th[tap], tl[tap], pack2(va.x, vb.x), pack2(va.y, vb.y), hs[b], ls[b]);
         }
       }
-      const long long idx = ((long long)a1 * g.ncx + a2) * Y + slot;
-      const double qv = f32_to_f64(hs) + f32_to_f64(ls);
-      q[idx] = qv;
-      acc[0] = fma(p[idx], qv, acc[0]);
+#pragma unroll
+      for (int b = 0; b < kClsCells; ++b) {
+        float h2[2], l2[2];
+        unpack2(hs[b / 2], h2[0], h2[1]);
+        unpack2(ls[b / 2], l2[0], l2[1]);
+        if (ok[b]) {
+          const double qv = f32_to_f64(h2[b & 1]) + f32_to_f64(l2[b & 1]);
+          q[idx + b * step] = qv;
+          acc[0] = fma(pv[b], qv, acc[0]);
+        }
+      }
     }
+    if (++sl == kClsStages) {
+      sl = 0;
+      ph ^= 1;
+    }
+    __syncthreads();
   }
   double tot[1];
   if (grid_sum_last<1>(acc, partials, counter, tot) && threadIdx.x == 0) {
@@ -946,26 +1037,34 @@ __global__ void __launch_bounds__(kThreads) k_matvec_pq_pairs_tiled(Geo g, const
   }
 }
 
-bool matvec_tiled_fits(const Geo& g) {
-  return g.p == 2 && g.n * g.Ypad <= kTiledMaxClasses && g.Ypad <= kThreads && g.nxi >= g.n;
+// column groups of the register-table form: the cell's n columns in ncg groups of CW, CW Ypad
+// threads each; Ypad at most 64 (the copies start one column before the vector, inside its guard band)
+bool matvec_cls_shape(const Geo& g, int* CW, int* ncg) {
+  const int most = kClsThreads / g.Ypad;
+  if (g.p != 2 || most < 2) return false;
+  *ncg = (g.n + most - 1) / most;
+  *CW = (g.n + *ncg - 1) / *ncg;
+  return (long long)g.n * *ncg <= kMaxRedBlocks;   // one block per plane residue and group at least
 }
 
 void launch_matvec_pq_pairs(dd_ctx* c, cudaStream_t s) {
   const Geo& g = c->g;
   if (g.p != 2) throw Error(DD_EINVAL, "the float-pair matvec pass is the p = 2 form");
-  if (c->matvec_tiled && matvec_tiled_fits(g)) {
-    const int TA = kThreads / g.Ypad;
-    const size_t smem = sizeof(float2) * ((size_t)g.n * g.Ypad * kPairTapStride3 + 3 * (size_t)(TA + 2) * g.Ypad + 2);
+  int CW = 0, ncg = 0;
+  if (c->matvec_tiled && matvec_cls_shape(g, &CW, &ncg)) {
+    const int threads = (CW * g.Ypad + 31) / 32 * 32;
+    const size_t smem = sizeof(float2) * kClsStages * kClsCells * (size_t)cls_cell_len(CW, g.Ypad);
     static PerDeviceOnce attr;
     once_per_device(attr, [] {
-      DD_CUDA(cudaFuncSetAttribute(k_matvec_pq_pairs_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+      DD_CUDA(cudaFuncSetAttribute(k_matvec_pq_pairs_cls, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     });
     int per_sm = 0;
-    DD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_matvec_pq_pairs_tiled, kThreads, smem));
-    const int nbr = std::max(1, 152 * std::max(per_sm, 1) / g.n);   // blocks per residue
-    launch_chain(k_matvec_pq_pairs_tiled, dim3(g.n * nbr), dim3(kThreads), smem, s, c->pdl != 0, g,
+    DD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_matvec_pq_pairs_cls, threads, smem));
+    const int groups = g.n * ncg, items = g.L * ((g.L + kClsCells - 1) / kClsCells);
+    const int nbr = std::max(1, std::min({152 * std::max(per_sm, 1) / groups, items, kMaxRedBlocks / groups}));
+    launch_chain(k_matvec_pq_pairs_cls, dim3(groups * nbr), dim3(threads), smem, s, c->pdl != 0, g,
                  (const float2*)c->tabS2, (const float2*)c->p2, c->pb[0], c->pb[1], c->q, c->st, c->red,
-                 c->cnt + CNT_PQ);
+                 c->cnt + CNT_PQ, CW, ncg, c->dev_err + 8);
     return;
   }
   launch_chain(k_matvec_pq_pairs, dim3(resident_grid(k_matvec_pq_pairs, interior_work(g), kThreads)), dim3(kThreads),
