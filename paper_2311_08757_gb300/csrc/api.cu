@@ -450,7 +450,6 @@ int pcg_run(dd_ctx* c, const double* b, double rtol, int maxit, int* iters, doub
 // in, solution out); stop when the true residual is <= rtol ||b - A x_0||.
 int gmres_run(dd_ctx* c, const double* b, double rtol, int maxit, int* iters, double* relres) {
   cudaStream_t s = c->stream;
-  const Geo& g = c->g;
   const int m = c->gm_restart;
   const int ld = m + 1;
   if (c->gm_alloc != m) {
@@ -464,7 +463,7 @@ int gmres_run(dd_ctx* c, const double* b, double rtol, int maxit, int* iters, do
     c->gm_Zptr = (double**)dev_alloc(c, sizeof(double*) * m);
     DD_CUDA(cudaMemcpyAsync(c->gm_Vptr, c->gm_V.data(), sizeof(double*) * (m + 1), cudaMemcpyHostToDevice, s));
     DD_CUDA(cudaMemcpyAsync(c->gm_Zptr, c->gm_Z.data(), sizeof(double*) * m, cudaMemcpyHostToDevice, s));
-    c->gm_part = (double*)dev_alloc(c, sizeof(double) * (size_t)(m + 1) * 304);
+    c->gm_part = (double*)dev_alloc(c, sizeof(double) * (size_t)(m + 1) * 152);
     c->gm_h = (double*)dev_alloc(c, sizeof(double) * (2 * ld + 1));
     c->gm_H = (double*)dev_alloc(c, sizeof(double) * (size_t)ld * m);
     c->gm_cs = (double*)dev_alloc(c, sizeof(double) * m);
@@ -473,12 +472,11 @@ int gmres_run(dd_ctx* c, const double* b, double rtol, int maxit, int* iters, do
     c->gm_y = (double*)dev_alloc(c, sizeof(double) * m);
     c->gm_res = (double*)dev_alloc(c, sizeof(double) * 2);
     DD_CUDA(cudaMallocHost(&c->gm_res_h, sizeof(double) * 2));
+    for (cudaEvent_t& e : c->gm_ev) DD_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     c->gm_alloc = m;
   }
   double* W = c->gm_W;
-  double* h2 = c->gm_h + ld;        // second Gram-Schmidt pass
-  double* nrm2 = c->gm_h + 2 * ld;  // ||w||^2
-  const double* const* Vp = c->gm_Vptr;
+  double* nrm2 = c->gm_h + 2 * ld;  // ||w||^2 (the two passes' projections before it)
   auto read_scalar = [&](const double* d) -> double {
     DD_CUDA(cudaMemcpyAsync(c->gm_res_h, d, sizeof(double), cudaMemcpyDeviceToHost, s));
     DD_CUDA(cudaStreamSynchronize(s));
@@ -494,7 +492,7 @@ int gmres_run(dd_ctx* c, const double* b, double rtol, int maxit, int* iters, do
   TIMED(KC_XRUPDATE, s, launch_dot(c, W, W, nrm2, s));
   const double r0 = std::sqrt(read_scalar(nrm2));
   int its = 0;
-  double rel = 0.0;
+  double rel = 0.0, est = r0, rate = 1.0;   // residual estimate and its last reduction
   if (!std::isfinite(r0)) return fail(c, DD_ENAN, "non-finite GMRES residual");
   if (r0 == 0.0) {
     if (iters) *iters = 0;
@@ -504,21 +502,48 @@ int gmres_run(dd_ctx* c, const double* b, double rtol, int maxit, int* iters, do
   while (true) {
     TIMED(KC_XRUPDATE, s, launch_scale_by_norm(c, W, nrm2, c->gm_V[0], s));
     TIMED(KC_MISC, s, launch_gmres_start(c, nrm2, s));
-    int j = 0, done = 0;
-    for (j = 0; j < m; ++j) {
+    // Step j: z_j = M^{-1} v_j, w = A z_j orthogonalised against v_0 .. v_j, v_{j+1} = w / ||w||.  The
+    // rotation of the Hessenberg column and the residual estimate's copy run on the side stream,
+    // beside the next step's first kernels.
+    auto step = [&](int j) {
       precond(c, c->gm_V[j], 0, c->gm_Z[j]);
       TIMED(KC_STENCIL, s, launch_stencil(c, c->tabS, c->gm_Z[j], W, s));
-      TIMED(KC_XRUPDATE, s, launch_multidot(c, j + 1, Vp, W, c->gm_h, 0, s));
-      TIMED(KC_XRUPDATE, s, launch_multiaxpy(c, j + 1, Vp, c->gm_h, -1.0, W, s));
-      TIMED(KC_XRUPDATE, s, launch_multidot(c, j + 1, Vp, W, h2, 0, s));
-      TIMED(KC_XRUPDATE, s, launch_multiaxpy(c, j + 1, Vp, h2, -1.0, W, s));
-      TIMED(KC_XRUPDATE, s, launch_add_inplace(c, j + 1, c->gm_h, h2, s));
-      TIMED(KC_XRUPDATE, s, launch_dot(c, W, W, nrm2, s));
+      TIMED(KC_XRUPDATE, s, launch_gm_orthogonalise(c, j, W, nrm2, s));
+      DD_CUDA(cudaEventRecord(c->ev_fork, s));
+      DD_CUDA(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
       TIMED(KC_XRUPDATE, s, launch_scale_by_norm(c, W, nrm2, c->gm_V[j + 1], s));
-      TIMED(KC_MISC, s, launch_givens(c, j, s));
-      const double est = read_scalar(c->gm_res);
+      TIMED(KC_MISC, c->side, launch_givens(c, j, c->gm_res + (j & 1), c->side));
+      DD_CUDA(cudaMemcpyAsync(c->gm_res_h + (j & 1), c->gm_res + (j & 1), sizeof(double), cudaMemcpyDeviceToHost,
+                              c->side));
+      DD_CUDA(cudaEventRecord(c->gm_ev[j & 1], c->side));
+    };
+    // The host issues step j + 1 before it waits for the estimate of step j, so the GPU does not
+    // idle over the read and the launches; a step too many only writes vectors and a column
+    // that the solution does not use.  Not after the first step of a solve and not when the
+    // last reduction, repeated, would end it.
+    int j = 0, done = 0, issued = 0;
+    for (j = 0; j < m; ++j) {
+      if (issued <= j) {
+        step(j);
+        issued = j + 1;
+      }
+      if (!c->timing && its > 0 && est * rate > rtol * r0 && j + 1 < m && its + 1 < maxit) {
+        step(j + 1);
+        issued = j + 2;
+      }
+      DD_CUDA(cudaEventSynchronize(c->gm_ev[j & 1]));
+      if (c->timing) {
+        DD_CUDA(cudaStreamSynchronize(s));
+        timer_collect(c);
+      }
+      rate = c->gm_res_h[j & 1] / est;
+      est = c->gm_res_h[j & 1];
       ++its;
-      if (!std::isfinite(est)) return fail(c, DD_ENAN, "non-finite GMRES residual");
+      if (!std::isfinite(est)) {
+        DD_CUDA(cudaStreamSynchronize(c->side));
+        DD_CUDA(cudaStreamSynchronize(s));
+        return fail(c, DD_ENAN, "non-finite GMRES residual");
+      }
       rel = est / r0;
       if (est <= rtol * r0) {
         done = 1;
@@ -530,6 +555,7 @@ int gmres_run(dd_ctx* c, const double* b, double rtol, int maxit, int* iters, do
         break;
       }
     }
+    DD_CUDA(cudaStreamWaitEvent(s, c->gm_ev[(issued - 1) & 1], 0));   // the last rotation issued
     const int mm = std::min(j, m);
     TIMED(KC_MISC, s, launch_backsolve(c, mm, s));
     TIMED(KC_XRUPDATE, s, launch_multiaxpy(c, mm, c->gm_Zptr, c->gm_y, 1.0, c->x, s));
@@ -595,6 +621,8 @@ void dd_destroy(dd_ctx* c) {
   for (void* p : c->allocs) cudaFree(p);
   if (c->st_h) cudaFreeHost(c->st_h);
   if (c->gm_res_h) cudaFreeHost(c->gm_res_h);
+  for (cudaEvent_t e : c->gm_ev)
+    if (e) cudaEventDestroy(e);
   if (c->ost_h) cudaFreeHost(c->ost_h);
   if (c->lst_h) cudaFreeHost(c->lst_h);
   if (c->side) cudaStreamDestroy(c->side);

@@ -218,6 +218,7 @@ struct dd_ctx {
   double** gm_Zptr = nullptr;
   double *gm_part = nullptr, *gm_h = nullptr, *gm_H = nullptr, *gm_cs = nullptr, *gm_sn = nullptr;
   double *gm_g = nullptr, *gm_y = nullptr, *gm_res = nullptr, *gm_res_h = nullptr;
+  cudaEvent_t gm_ev[2] = {};        // the estimate of an even (odd) step is on the host
   double* gout = nullptr;         // gradient staging (n_V doubles)
 
   // cell problem
@@ -420,15 +421,13 @@ void launch_dot(dd_ctx* c, const double* a, const double* b, double* out, cudaSt
 void launch_axpby(dd_ctx* c, double ca, const double* x, double cb_scale, const double* cb, const double* y,
                   double* out, cudaStream_t s);
 void launch_tab_shift(dd_ctx* c, double shift, double* dst);
-void launch_multidot(dd_ctx* c, int nv, const double* const* V, const double* w, double* h, int accumulate,
-                     cudaStream_t s);
+void launch_gm_orthogonalise(dd_ctx* c, int j, double* w, double* nrm2, cudaStream_t s);
 void launch_multiaxpy(dd_ctx* c, int nv, const double* const* V, const double* coef, double sign, double* w,
                       cudaStream_t s);
 void launch_scale_by_norm(dd_ctx* c, const double* w, const double* nrm2, double* v, cudaStream_t s);
-void launch_givens(dd_ctx* c, int j, cudaStream_t s);
+void launch_givens(dd_ctx* c, int j, double* res, cudaStream_t s);
 void launch_backsolve(dd_ctx* c, int m, cudaStream_t s);
 void launch_gmres_start(dd_ctx* c, const double* nrm2, cudaStream_t s);
-void launch_add_inplace(dd_ctx* c, int n, double* a, const double* b, cudaStream_t s);
 
 // ----- batched launchers (vmap[k] = {problem, block within the problem's launch}) -----
 void batch_grid_sizes(const dd_ctx* c, BInst* I);   // the nb_* of the plain launchers
