@@ -1194,58 +1194,41 @@ namespace {
 // of phi, where A - lambda M is positive definite even when lambda and phi carry the error
 // of the eigen-solve (there A - lambda M has a tiny negative eigenvalue along phi).
 // Polak-Ribiere beta (exact for the FP64 preconditioner, flexible for the rounded one).
-// Vectors: b (in, overwritten as the residual), x (out), u = M phi, phi; scratch p, q, rp.
+// Vectors: r (in, overwritten as the residual), x (out), u = M phi, phi; scratch p, q.  The scalars
+// stay on the device (k_adjoint.cu); the host looks at the done flag every kAdjCheck iterations,
+// whose launches it issues faster than the GPU runs them.
+constexpr int kAdjCheck = 8;
 int adjoint_pcg(dd_ctx* c, double* r, double* x, const double* u, const double* phi, double* p, double* q,
-                double* zs, double rtol, int maxit, int* iters) {
+                double rtol, int maxit, int* iters) {
   cudaStream_t s = c->stream;
   const Geo& g = c->g;
-  double* d = c->gscal;   // device scalars
-  auto dot = [&](const double* a, const double* b2) -> double {
-    launch_dot(c, a, b2, d, s);
-    double h = 0.0;
-    DD_CUDA(cudaMemcpyAsync(&h, d, sizeof(double), cudaMemcpyDeviceToHost, s));
-    DD_CUDA(cudaStreamSynchronize(s));
-    return h;
-  };
-  auto axpby = [&](double a, const double* xv, double bcoef, const double* yv, double* out) {
-    launch_axpby(c, a, xv, bcoef, nullptr, yv, out, s);
-  };
-  auto apply_prec = [&]() {   // zs = Pi M^{-1} Pi^T r  (r is kept orthogonal to phi)
-    PcgState init;
-    std::memset(&init, 0, sizeof(init));
-    DD_CUDA(cudaMemcpyAsync(c->st, &init, sizeof(init), cudaMemcpyHostToDevice, s));
-    precond(c, r, 0);
-    const double t = dot(u, c->z);
-    axpby(1.0, c->z, -t, phi, zs);
-  };
+  PcgState init;
+  std::memset(&init, 0, sizeof(init));
+  init.tol2 = rtol * rtol;
+  init.maxit = maxit;
+  DD_CUDA(cudaMemcpyAsync(c->st, &init, sizeof(init), cudaMemcpyHostToDevice, s));
   DD_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * g.plen, s));
-  const double rr0 = dot(r, r);
-  *iters = 0;
-  if (rr0 == 0.0) return DD_OK;
-  apply_prec();
-  DD_CUDA(cudaMemcpyAsync(p, zs, sizeof(double) * g.plen, cudaMemcpyDeviceToDevice, s));
-  double rz = dot(r, zs);
-  for (int k = 1; k <= maxit; ++k) {
-    TIMED(KC_STENCIL, s, launch_stencil(c, c->tabL, p, q, s));
-    const double pq = dot(p, q);
-    if (!(pq > 0.0)) return fail(c, std::isfinite(pq) ? DD_ENOTSPD : DD_ENAN, "adjoint: p^T (A - lambda M) p <= 0");
-    const double alpha = rz / pq;
-    axpby(1.0, x, alpha, p, x);
-    axpby(1.0, r, -alpha, q, r);
-    // keep r orthogonal to phi against drift
-    const double tp = dot(phi, r);
-    axpby(1.0, r, -tp, u, r);
-    const double rr = dot(r, r);
-    *iters = k;
-    if (rr <= rtol * rtol * rr0) return DD_OK;
-    apply_prec();
-    const double zq = dot(zs, q);
-    const double rz_new = dot(r, zs);
-    const double beta = -zq / pq;   // (z_{k+1}, r_{k+1} - r_k) / (z_k, r_k)
-    axpby(1.0, zs, beta, p, p);
-    rz = rz_new;
-  }
-  return fail(c, DD_EMAXIT, "adjoint PCG reached maxit");
+  DD_CUDA(cudaMemsetAsync(p, 0, sizeof(double) * g.plen, s));
+  TIMED(KC_MISC, s, launch_adj_init(c, r, phi, s));
+  precond(c, r, 0);
+  TIMED(KC_MISC, s, launch_adj_dots(c, u, r, q, 1, s));
+  do {
+    for (int k = 0; k < kAdjCheck; ++k) {
+      TIMED(KC_PUPDATE, s, launch_adj_pupdate(c, phi, p, s));
+      TIMED(KC_STENCIL, s, launch_adj_stencil(c, c->tabL, p, phi, q, s));
+      TIMED(KC_XRUPDATE, s, launch_adj_update(c, p, q, u, phi, x, r, s));
+      precond(c, r, 0);
+      TIMED(KC_MISC, s, launch_adj_dots(c, u, r, q, 0, s));
+    }
+    DD_CUDA(cudaMemcpyAsync(c->st_h, c->st, sizeof(PcgState), cudaMemcpyDeviceToHost, s));
+    DD_CUDA(cudaStreamSynchronize(s));
+    if (c->timing) timer_collect(c);
+  } while (!c->st_h->done);
+  *iters = c->st_h->iter;
+  const int status = c->st_h->status;
+  if (status == DD_EMAXIT) return fail(c, status, "adjoint PCG reached maxit");
+  if (status != 0) return fail(c, status, "adjoint: p^T (A - lambda M) p <= 0");
+  return DD_OK;
 }
 
 }  // namespace
@@ -1266,10 +1249,11 @@ int dd_potential_gradient(dd_ctx* c, const double* phi, double lambda, double g_
       for (double*& v : c->gv) v = alloc_vec(c);
       c->tabL = (double*)dev_alloc(c, sizeof(double) * (size_t)g.ncls * g.ntap);
       c->gscal = (double*)dev_alloc(c, sizeof(double) * 2);
+      c->adj = (AdjScal*)dev_alloc(c, sizeof(AdjScal));
       c->gout = (double*)dev_alloc(c, sizeof(double) * nV);
     }
     double *PHI = c->gv[0], *G = c->gv[1], *U = c->gv[2], *VV = c->gv[3];
-    double *W = c->gv[4], *P = c->gv[5], *Q = c->gv[6], *Z = c->gv[7];
+    double *W = c->gv[4], *P = c->gv[5], *Q = c->gv[6];
     load_vec(c, phi, PHI);
     int iters = 0;
     if (g_phi) {
@@ -1279,7 +1263,7 @@ int dd_potential_gradient(dd_ctx* c, const double* phi, double lambda, double g_
       TIMED(KC_OUTER, s, launch_dot(c, PHI, G, c->gscal, s));
       TIMED(KC_OUTER, s, launch_axpby(c, 1.0, G, -1.0, c->gscal, U, G, s));
       launch_tab_shift(c, lambda, c->tabL);
-      const int prc = adjoint_pcg(c, G, W, U, PHI, P, Q, Z, rtol, 10000, &iters);
+      const int prc = adjoint_pcg(c, G, W, U, PHI, P, Q, rtol, 10000, &iters);
       if (prc != DD_OK) return prc;
       // w <- w - phi (M phi)^T w (the iterates stay there up to rounding)
       TIMED(KC_OUTER, s, launch_dot(c, U, W, c->gscal, s));

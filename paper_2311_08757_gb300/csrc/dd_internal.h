@@ -117,6 +117,13 @@ struct LopState {
   int m, status;
 };
 
+// Scalars of the adjoint solve's projections (k_adjoint.cu).
+struct AdjScal {
+  double t;          // (M phi, z)
+  double tp;         // (phi, r - alpha q)
+  double phr, phq;   // (phi, r), (phi, q)
+};
+
 // Scalars of the outer iteration.
 struct OuterState {
   double wMw, wsum, scale;
@@ -207,8 +214,9 @@ struct dd_ctx {
   double* tabL = nullptr;   // K + M_V - lambda M (adjoint of the eigenvector)
   double* qp_part = nullptr;      // quadrature-point reduction partials
   long long qp_part_len = 0;
-  double* gv[8] = {};             // gradient work vectors
+  double* gv[7] = {};             // gradient work vectors
   double* gscal = nullptr;        // device scalars of the gradient projections
+  dd::AdjScal* adj = nullptr;     // and of the adjoint solve
   // GMRES (restart gm_restart): basis V[0..m], preconditioned directions Z[0..m-1]
   int krylov = 0;                 // inner solver of the eigen-iterations: 0 PCG, 1 GMRES
   int gm_restart = 30, gm_alloc = 0;
@@ -421,6 +429,12 @@ void launch_dot(dd_ctx* c, const double* a, const double* b, double* out, cudaSt
 void launch_axpby(dd_ctx* c, double ca, const double* x, double cb_scale, const double* cb, const double* y,
                   double* out, cudaStream_t s);
 void launch_tab_shift(dd_ctx* c, double shift, double* dst);
+void launch_adj_init(dd_ctx* c, const double* r, const double* phi, cudaStream_t s);
+void launch_adj_pupdate(dd_ctx* c, const double* phi, double* p, cudaStream_t s);
+void launch_adj_stencil(dd_ctx* c, const double* tab, const double* p, const double* phi, double* q, cudaStream_t s);
+void launch_adj_update(dd_ctx* c, const double* p, const double* q, const double* u, const double* phi, double* x,
+                       double* r, cudaStream_t s);
+void launch_adj_dots(dd_ctx* c, const double* u, const double* r, const double* q, int start, cudaStream_t s);
 void launch_gm_orthogonalise(dd_ctx* c, int j, double* w, double* nrm2, cudaStream_t s);
 void launch_multiaxpy(dd_ctx* c, int nv, const double* const* V, const double* coef, double sign, double* w,
                       cudaStream_t s);
