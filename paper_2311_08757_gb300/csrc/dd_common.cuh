@@ -168,6 +168,54 @@ __device__ __forceinline__ bool grid_sum_last(double (&v)[NV], double* partials,
   return grid_sum_last<NV>(v, partials, counter, tot, vblk_self());
 }
 
+// grid_sum_last of blocks of 256 threads by blocks of 128: thread t holds the values of threads 2 t
+// (x) and 2 t + 1 (y); every addition is the one made there, in the same order.
+template <int NV>
+__device__ __forceinline__ void block_sum_pairs(const double2 (&v)[NV], double (&out)[NV]) {
+  __shared__ __align__(16) double st[NV][256];
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) *reinterpret_cast<double2*>(&st[k][2 * threadIdx.x]) = v[k];
+  __syncthreads();
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      double a = st[k][lane];
+      for (int w = 1; w < 8; ++w) a += st[k][lane + 32 * w];
+      out[k] = warp_sum(a);
+    }
+  }
+  __syncthreads();
+}
+template <int NV>
+__device__ __forceinline__ bool grid_sum_last_pairs(const double2 (&v)[NV], double* partials, unsigned* counter,
+                                                    double (&tot)[NV], VBlk vb) {
+  __shared__ int s_last;
+  double b[NV];
+  block_sum_pairs<NV>(v, b);
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) partials[(size_t)k * kMaxRedBlocks + vb.b] = b[k];
+    __threadfence();
+    s_last = (atomicAdd(counter, 1u) == (unsigned)vb.nb - 1);
+  }
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  double2 s[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    s[k] = make_double2(0.0, 0.0);
+    for (int e = 2 * threadIdx.x; e < vb.nb; e += 256) {
+      s[k].x += __ldcg(partials + (size_t)k * kMaxRedBlocks + e);
+      if (e + 1 < vb.nb) s[k].y += __ldcg(partials + (size_t)k * kMaxRedBlocks + e + 1);
+    }
+  }
+  block_sum_pairs<NV>(s, tot);
+  if (threadIdx.x == 0) *counter = 0u;
+  return true;
+}
+
 // ---- precision conversions on the integer pipe ------------------------------------------
 // GB300 retires FP64 instructions (conversions included) at 2 per clock per SM; these
 // conversions do the same rounding with integer operations for normal-range values.

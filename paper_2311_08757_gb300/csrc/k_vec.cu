@@ -1186,17 +1186,23 @@ __device__ __forceinline__ double to_f64(double d) { return d; }
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
 
-// Register budget: 32 per thread (8 blocks of 256 per SM) for p = 1, which fits it; 48
-// (5 blocks) for p = 2, whose four owners per node spilled at 32 (on the L = 64, h = 1/16
-// three-dimensional box: 987 -> 971 ms per ground state).  The FP64 p = 1 variant spills a
-// little at 32 yet ran 4% faster there than at 48 without spills.
+// A thread takes two neighbouring slots of one node column: they share the owners and the table
+// loads, and r, q, z, the local results and the weights move in pairs; an absent owner costs
+// predicated-off loads only.  Blocks of 128 threads at 64 registers, 8 per SM.  The two slots' dot
+// products are summed apart and added up as blocks of 256 threads with one slot each would
+// (grid_sum_last_pairs): p = 1 solves of long boxes amplify a change of that order.  One slot per
+// thread, every owner's loads made and masked: L = 64, h = 1/16 (p = 2) 149 -> 89 us, its streams
+// alone 73; p = 1, L = 2048, h = 1/32 19.9 -> 18.3 us (FP64 local solves 37.0 -> 32.6), L = 256
+// 9.4 -> 8.3 us: the two dot products' FP64 instructions and the table's round trip remain.
 // ARITH (p = 1): the owners from p1_owners and their packed rows from the subdomain index
 // (subdomain i is packed row i; its type is pt.x, pt.y or pt.z for the left end, the interior
 // and the right end) instead of the two index tables -- the same values, without two levels of
 // dependent loads per node (the host checks the formula against the tables at set-up).
 // UPD (p = 1 iterations whose x update ran in the packing, launch_pack_xr): r_out = r - alpha q
 // first (the same FMA as the separate x/r update, each node once), and the dots take that r.
-template <int P, typename TY, bool RAS, int U, bool ARITH = false, bool UPD = false>
+__device__ __forceinline__ float2 ldg2(const float* p) { return __ldg(reinterpret_cast<const float2*>(p)); }
+__device__ __forceinline__ double2 ldg2(const double* p) { return __ldg(reinterpret_cast<const double2*>(p)); }
+template <int P, typename TY, bool RAS, bool ARITH = false, bool UPD = false>
 __device__ __forceinline__ void prolong_body(VBlk vb, Geo g, const int4* __restrict__ axown,
                                                       const int4* __restrict__ subrow,
                                                       const int4* __restrict__ colrow, const TY* __restrict__ Y,
@@ -1214,89 +1220,86 @@ __device__ __forceinline__ void prolong_body(VBlk vb, Geo g, const int4* __restr
   if (mode != 0 && st->done) return;
   const bool flex = (mode == 2) && st->flexible;
   const double alpha_r = UPD ? st->alpha : 0.0;
-  const long long total = (long long)g.nxi * (P == 2 ? g.nxi : 1) * g.Ypad;
-  const long long stride = (long long)vb.nb * blockDim.x;
-  constexpr int NO = (P == 2) ? 4 : 2;  // owners per node at most; U nodes per thread and pass
-  double acc[2] = {0.0, 0.0};
-  for (long long t0 = (long long)vb.b * blockDim.x + threadIdx.x; t0 < total; t0 += U * stride) {
-    // branch-free: out-of-range nodes and absent owners read valid addresses and are masked
-    bool in[U], valid[U];
-    Node nd[U];
-    int4 A1[U], A2[U], CR[U];
+  const long long total = (long long)g.nxi * (P == 2 ? g.nxi : 1) * g.Ypad / 2;   // pairs of slots
+  constexpr int NO = (P == 2) ? 4 : 2;  // owners per node at most
+  using TY2 = decltype(ldg2((const TY*)nullptr));
+  double2 acc[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};   // the two slots' sums apart
+  for (long long t = (long long)vb.b * blockDim.x + threadIdx.x; t < total; t += (long long)vb.nb * blockDim.x) {
+    const Node nd = node_of<P>(g, 2 * t);
+    const bool valid0 = nd.slot < g.nyi, valid1 = nd.slot + 1 < g.nyi;
+    double2 rv = make_double2(0.0, 0.0), qv = rv;
+    if (mode != 0) rv = *reinterpret_cast<const double2*>(r + nd.idx);
+    if (flex || UPD) qv = *reinterpret_cast<const double2*>(q + nd.idx);
+    const int4 A1 = ARITH ? p1_owners(g, nd.a1) : __ldg(axown + nd.a1);
+    const int4 A2 = (P == 2) ? __ldg(axown + nd.a2) : make_int4(0, 0, -1, 0);
+    const int4 CR = kColRow ? __ldg(colrow + nd.a1) : make_int4(0, 0, 0, 0);
+    bool ok[NO];
+    int sub[NO];
+    size_t ry[NO], rw[NO];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const long long t = t0 + u * stride;
-      in[u] = t < total;
-      nd[u] = node_of<P>(g, in[u] ? t : 0);
-      valid[u] = in[u] && nd[u].slot < g.nyi;
-      A1[u] = ARITH ? p1_owners(g, nd[u].a1) : __ldg(axown + nd[u].a1);
-      A2[u] = (P == 2) ? __ldg(axown + nd[u].a2) : make_int4(0, 0, -1, 0);
-      CR[u] = kColRow ? __ldg(colrow + nd[u].a1) : make_int4(0, 0, 0, 0);
+    for (int e = 0; e < NO; ++e) {
+      const int i = (P == 2) ? e >> 1 : e, k = (P == 2) ? e & 1 : 0;
+      const int o1 = i ? A1.z : A1.x, l1 = i ? A1.w : A1.y;
+      const int o2 = k ? A2.z : A2.x, l2 = k ? A2.w : A2.y;
+      ok[e] = o1 >= 0 && (P == 1 || o2 >= 0);
+      sub[e] = ok[e] ? ((P == 1) ? o1 : o1 * g.L + o2) : 0;
+      int4 sr = make_int4(0, 0, 1, 0);
+      int loc = nd.slot;
+      if (kColRow) {   // the owner's packed row and type row, its local column included
+        sr.x = i ? CR.z : CR.x;
+        sr.y = i ? CR.w : CR.y;
+      } else if (ARITH) {
+        const int sb = sub[e], ty = sb == 0 ? pt.x : (sb == g.L - 1 ? pt.z : pt.y);
+        sr.x = sb * kpad;
+        sr.y = ty * kpad;
+        loc += l1 * g.Ypad;
+      } else if (ok[e]) {
+        sr = __ldg(subrow + sub[e]);
+        loc += (P == 1 ? l1 : l1 * sr.z + l2) * g.Ypad;
+      }
+      ry[e] = (size_t)sr.x + loc;
+      rw[e] = (size_t)sr.y + loc;
     }
-    bool ok[U][NO];
-    int sub[U][NO], loc[U][NO];
-    int4 sr[U][NO];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int e = 0; e < NO; ++e) {
-        const int i = (P == 2) ? e >> 1 : e, k = (P == 2) ? e & 1 : 0;
-        const int o1 = i ? A1[u].z : A1[u].x, l1 = i ? A1[u].w : A1[u].y;
-        const int o2 = k ? A2[u].z : A2[u].x, l2 = k ? A2[u].w : A2[u].y;
-        ok[u][e] = o1 >= 0 && (P == 1 || o2 >= 0);
-        sub[u][e] = ok[u][e] ? ((P == 1) ? o1 : o1 * g.L + o2) : 0;
-        if (kColRow) {   // the owner's packed row and type row, its local column included
-          sr[u][e] = i ? make_int4(CR[u].z, CR[u].w, 1, 0) : make_int4(CR[u].x, CR[u].y, 1, 0);
-          loc[u][e] = ok[u][e] ? nd[u].slot : 0;
-          continue;
-        }
-        if (ARITH) {
-          const int sb = sub[u][e];
-          const int ty = sb == 0 ? pt.x : (sb == g.L - 1 ? pt.z : pt.y);
-          sr[u][e] = make_int4(sb * kpad, ty * kpad, 1, 0);
-        } else {
-          sr[u][e] = __ldg(subrow + sub[u][e]);
-        }
-        loc[u][e] = ok[u][e] ? (((P == 1) ? l1 : l1 * sr[u][e].z + l2) * g.Ypad + nd[u].slot) : 0;
-      }
-    double rv[U], qv[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      rv[u] = (mode != 0) ? r[nd[u].idx] : 0.0;
-      const double qq = (flex || UPD) ? q[nd[u].idx] : 0.0;
-      if (UPD) {
-        rv[u] = fma(-alpha_r, qq, rv[u]);
-        if (in[u]) r_out[nd[u].idx] = rv[u];
-      }
-      qv[u] = flex ? qq : 0.0;
+    if (UPD) {
+      rv.x = fma(-alpha_r, qv.x, rv.x);
+      rv.y = fma(-alpha_r, qv.y, rv.y);
+      *reinterpret_cast<double2*>(r_out + nd.idx) = rv;
     }
+    TY ysx = (TY)0, ysy = (TY)0, czx = (TY)0, czy = (TY)0;
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      TY ys = (TY)0, cz = (TY)0;
-#pragma unroll
-      for (int e = 0; e < NO; ++e) {
-        const size_t ry = (size_t)sr[u][e].x + loc[u][e], rw = (size_t)sr[u][e].y + loc[u][e];
-        TY y = Y[ry];
-        if (RAS) y = __ldg(puT + rw) * y;   // R_i^T D_i y_i
-        const TY cw = coarse ? fma_t(__ldg(wT + rw), __ldg(u0 + sub[u][e]), cz) : cz;
-        if (ok[u][e]) {
-          ys += y;
-          cz = cw;
+    for (int e = 0; e < NO; ++e)
+      if (ok[e]) {
+        TY2 y = ldg2(Y + ry[e]);
+        if (RAS) {   // R_i^T D_i y_i
+          const TY2 d = ldg2(puT + rw[e]);
+          y.x = d.x * y.x;
+          y.y = d.y * y.y;
+        }
+        ysx += y.x;
+        ysy += y.y;
+        if (coarse) {
+          const TY2 w = ldg2(wT + rw[e]);
+          const TY u = __ldg(u0 + sub[e]);
+          czx = fma_t(w.x, u, czx);
+          czy = fma_t(w.y, u, czy);
         }
       }
-      const double v = valid[u] ? to_f64(ys + cz) : 0.0;
-      if (in[u]) {
-        z[nd[u].idx] = v;
-        if (mode != 0) {
-          acc[0] = fma(rv[u], v, acc[0]);
-          if (flex) acc[1] = fma(qv[u], v, acc[1]);
-        }
+    double2 v;
+    v.x = valid0 ? to_f64(ysx + czx) : 0.0;
+    v.y = valid1 ? to_f64(ysy + czy) : 0.0;
+    *reinterpret_cast<double2*>(z + nd.idx) = v;
+    if (mode != 0) {
+      acc[0].x = fma(rv.x, v.x, acc[0].x);
+      acc[0].y = fma(rv.y, v.y, acc[0].y);
+      if (flex) {
+        acc[1].x = fma(qv.x, v.x, acc[1].x);
+        acc[1].y = fma(qv.y, v.y, acc[1].y);
       }
     }
   }
   if (mode == 0) return;
   double tot[2];
-  if (grid_sum_last<2>(acc, partials, counter, tot, vb) && threadIdx.x == 0) {
+  if (grid_sum_last_pairs<2>(acc, partials, counter, tot, vb) && threadIdx.x == 0) {
     const double rz = tot[0];
     if (!isfinite(rz)) {
       st->status = DD_ENAN;
@@ -1315,8 +1318,9 @@ __device__ __forceinline__ void prolong_body(VBlk vb, Geo g, const int4* __restr
   }
 }
 
-template <int P, typename TY, bool RAS, int U, bool ARITH = false, bool UPD = false>
-__global__ void __launch_bounds__(kThreads, (P == 1 ? 8 : 5) / U) k_prolong(Geo g, const int4* __restrict__ axown,
+constexpr int kProlongThreads = kThreads / 2, kProlongBlocks = 8;   // per block, per SM
+template <int P, typename TY, bool RAS, bool ARITH = false, bool UPD = false>
+__global__ void __launch_bounds__(kProlongThreads, kProlongBlocks) k_prolong(Geo g, const int4* __restrict__ axown,
                                                       const int4* __restrict__ subrow,
                                                       const int4* __restrict__ colrow, const TY* __restrict__ Y,
                                                       const TY* __restrict__ wT, const TY* __restrict__ puT,
@@ -1326,25 +1330,20 @@ __global__ void __launch_bounds__(kThreads, (P == 1 ? 8 : 5) / U) k_prolong(Geo 
                                                       double* partials, unsigned* counter, int kpad, int4 pt,
                                                       double* r_out) {
   pdl_enter();
-  prolong_body<P, TY, RAS, U, ARITH, UPD>(vblk_self(), g, axown, subrow, colrow, Y, wT, puT, u0, coarse, r, q, z,
+  prolong_body<P, TY, RAS, ARITH, UPD>(vblk_self(), g, axown, subrow, colrow, Y, wT, puT, u0, coarse, r, q, z,
                                           mode, st, partials, counter, kpad, pt, r_out);
 }
 
-// nodes per thread and pass (each node's loads go out together, absent owners masked):
-// measured on the L = 2048, h = 1/32 box, 24.7 / 31.5 / 42.4 us per launch for 1 / 2 / 4 (the register cost of
-// more nodes takes away more resident warps than it adds loads in flight)
-constexpr int kProlongU = 1;
-
 void launch_prolong(dd_ctx* c, int mode, cudaStream_t s, double* zout, bool upd) {
   const Geo& g = c->g;
-  const long long work = interior_work(g);
+  const long long work = interior_work(g) / 2;
   const int coarse = c->grid.coarse;
   const bool f32 = (c->grid.precision != DD_PREC_FP64);
   double* z = zout != nullptr ? zout : c->z;
   const bool upd_r = upd && mode == 2;
 #define DD_PROLONG_A(PP, TY, YP, W, PU, U0, RS, AR, UP)                                                          \
-  launch_chain(k_prolong<PP, TY, RS, kProlongU, AR, UP>,                                                          \
-               dim3(resident_grid(k_prolong<PP, TY, RS, kProlongU, AR, false>, work, kThreads)), dim3(kThreads), 0, \
+  launch_chain(k_prolong<PP, TY, RS, AR, UP>,                                                          \
+               dim3(grid_blocks(work, kProlongThreads, kProlongBlocks)), dim3(kProlongThreads), 0, \
                s, c->pdl != 0, g, (const int4*)c->axown, (const int4*)c->subrow, (const int4*)c->colrow,        \
                (const TY*)(YP),                                                                               \
                (const TY*)(W), (const TY*)(PU), (const TY*)(U0), coarse, (const double*)c->r,                    \
@@ -1712,12 +1711,12 @@ __global__ void __launch_bounds__(kThreads) kb_xr_update(const BInst* __restrict
 }
 
 template <bool ARITH, bool UPD>
-__global__ void __launch_bounds__(kThreads, 8 / kProlongU) kb_prolong(const BInst* __restrict__ B,
-                                                                      const int2* __restrict__ vmap, int mode) {
+__global__ void __launch_bounds__(kProlongThreads, kProlongBlocks) kb_prolong(const BInst* __restrict__ B,
+                                                                 const int2* __restrict__ vmap, int mode) {
   const int2 m = vmap[blockIdx.x];
   const BInst& I = B[m.x];
   if (!I.active) return;
-  prolong_body<1, float, false, kProlongU, ARITH, UPD>(VBlk{m.y, I.nb_prolong}, I.g, I.axown, I.subrow, I.colrow, I.Y32,
+  prolong_body<1, float, false, ARITH, UPD>(VBlk{m.y, I.nb_prolong}, I.g, I.axown, I.subrow, I.colrow, I.Y32,
                                                        I.wT32, I.puT32, I.u0f, I.coarse, I.r, I.q, I.z, mode, I.st,
                                                        I.red, I.cnt + CNT_RZ, I.kpad, I.ptypes, UPD ? I.r : nullptr);
 }
@@ -1860,8 +1859,7 @@ void batch_grid_sizes(const dd_ctx* c, BInst* I) {
   I->nb_init = grid_blocks(w, kThreads);
   I->nb_fused = ntiles < 152 * 6 ? ntiles : 152 * 6;
   I->nb_xr = xr_blocks(c);
-  I->nb_prolong = c->prolong_arith ? resident_grid(k_prolong<1, float, false, kProlongU, true>, w, kThreads)
-                                    : resident_grid(k_prolong<1, float, false, kProlongU, false>, w, kThreads);
+  I->nb_prolong = grid_blocks(w / 2, kProlongThreads, kProlongBlocks);
   I->nb_sdot = resident_grid(k_stencil<1, true>, w, kThreads);
   I->nb_st = resident_grid(k_stencil<1, false>, w, kThreads);
   I->nb_vec = grid_blocks(g.plen, kThreads);
@@ -1930,11 +1928,11 @@ void launch_b_xr_update(const BInst* B, const int2* vmap, int nvb, cudaStream_t 
 
 void launch_b_prolong(const BInst* B, const int2* vmap, int nvb, int mode, bool arith, bool upd, cudaStream_t s) {
   if (upd && mode == 2) {
-    if (arith) (kb_prolong<true, true><<<nvb, kThreads, 0, s>>>(B, vmap, mode), dd::note_launch());
-    else (kb_prolong<false, true><<<nvb, kThreads, 0, s>>>(B, vmap, mode), dd::note_launch());
+    if (arith) (kb_prolong<true, true><<<nvb, kProlongThreads, 0, s>>>(B, vmap, mode), dd::note_launch());
+    else (kb_prolong<false, true><<<nvb, kProlongThreads, 0, s>>>(B, vmap, mode), dd::note_launch());
   } else {
-    if (arith) (kb_prolong<true, false><<<nvb, kThreads, 0, s>>>(B, vmap, mode), dd::note_launch());
-    else (kb_prolong<false, false><<<nvb, kThreads, 0, s>>>(B, vmap, mode), dd::note_launch());
+    if (arith) (kb_prolong<true, false><<<nvb, kProlongThreads, 0, s>>>(B, vmap, mode), dd::note_launch());
+    else (kb_prolong<false, false><<<nvb, kProlongThreads, 0, s>>>(B, vmap, mode), dd::note_launch());
   }
   DD_CUDA(cudaGetLastError());
 }
