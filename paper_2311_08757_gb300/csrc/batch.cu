@@ -51,6 +51,7 @@ struct BGroup {
   int ypad = 0, precision = 0, check_every = 8;
   bool arith = true;               // every instance's prolong-sum owners in closed form
   bool pairs = false;              // q = A_sigma p in float pairs (the same choice for every instance)
+  bool lag = false;                // x updated one iteration late, by the p update (the same for every instance)
   bool fuse = false;               // the x/r update inside the packing (the same for every instance)
   dd::BGemm* gemm = nullptr;
   int bn = 0;                      // N tile of the grouped contraction (timed at build)
@@ -115,7 +116,7 @@ void free_group(BGroup* g) {
 long long option_signature(const dd_batch* b) {
   long long h = 1469598103934665603LL;
   for (const dd_ctx* c : b->ctx)
-    for (int v : {c->prolong_arith, c->pq_pairs, c->fuse_xr, c->flexible_opt, c->check_every, c->gemm_bn_opt})
+    for (int v : {c->prolong_arith, c->pq_pairs, c->fuse_xr, c->x_lag, c->flexible_opt, c->check_every, c->gemm_bn_opt})
       h = (h ^ (long long)(v + 7)) * 1099511628211LL;
   return h;
 }
@@ -186,12 +187,12 @@ void precond(BGroup* g, int mode, bool packed = false) {
 }
 
 void pcg_iteration(BGroup* g) {
-  dd::launch_b_fused_pq(g->B, g->vm_fused, g->n_fused, g->ypad, g->pairs, g->s);
+  dd::launch_b_fused_pq(g->B, g->vm_fused, g->n_fused, g->ypad, g->pairs, g->lag, g->s);
   if (g->fuse) {
     dd::launch_b_pack_xr(g->B, g->vm_pack, g->n_pack, g->precision, g->s);
     precond(g, 2, true);
   } else {
-    dd::launch_b_xr_update(g->B, g->vm_xr, g->n_xr, g->s);
+    dd::launch_b_xr_update(g->B, g->vm_xr, g->n_xr, g->lag, g->s);
     precond(g, 2);
   }
 }
@@ -265,6 +266,7 @@ BGroup* build_group(dd_batch* b, const std::vector<int>& idx) {
       I.pq_pairs = c->pq_pairs;
       g->pairs = c->pq_pairs != 0;
       g->fuse = c->fuse_xr != 0;
+      g->lag = c->x_lag != 0 && !g->fuse;
       I.st = c->st; I.ost = c->ost; I.red = c->red; I.cnt = c->cnt;
       I.subs = c->subs; I.slot_of_sub = c->slot_of_sub; I.Rpack = c->Rpack; I.wT = c->wT; I.c0 = c->c0;
       I.u0 = c->u0; I.u0f = c->u0f; I.Y32 = c->Y32; I.wT32 = c->wT32; I.puT32 = c->puT32;
@@ -470,6 +472,7 @@ int run_ipm(dd_batch* b, BGroup* g, const Ready& ready, const Outputs& o) {
         if (state[j] == ST_RUNNING && !g->stat_h[j].pcg_done) all = false;
       if (all) break;
     }
+    if (g->lag) launch_b_x_final(g->B, g->vm_vec, g->n_vec, g->s);
     for (int j = 0; j < m; ++j) {
       if (state[j] != ST_RUNNING) continue;
       inner[j] += g->stat_h[j].pcg_iter;

@@ -1130,23 +1130,29 @@ __global__ void __launch_bounds__(kThreads) k_xr_update(long long n, double* pb0
 
 // After the last PCG iteration K: x += alpha_K p_K, the update the lagged scheme left for a
 // next p update that does not run.  Not after a failed (p, q) or a non-finite iterate.
-__global__ void __launch_bounds__(kThreads) k_x_final(long long n, const double* __restrict__ pb0,
-                                                      const double* __restrict__ pb1, double* __restrict__ x,
-                                                      const PcgState* st) {
+__device__ __forceinline__ void x_final_body(VBlk vb, long long n, const double* __restrict__ pb0,
+                                             const double* __restrict__ pb1, double* __restrict__ x,
+                                             const PcgState* st) {
   if (st->status != 0 && st->status != DD_EMAXIT) return;
   const double alpha = st->alpha;
   // after iteration K the counter is K + 1, and p_K sits where iteration K + 1 would read p_{k-1}
   const double2* p2 = reinterpret_cast<const double2*>(p_prev(const_cast<double*>(pb0), const_cast<double*>(pb1),
                                                                 st->iter));
   double2* x2 = reinterpret_cast<double2*>(x);
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n / 2;
-       t += (long long)gridDim.x * blockDim.x) {
+  for (long long t = vb.b * (long long)blockDim.x + threadIdx.x; t < n / 2;
+       t += (long long)vb.nb * blockDim.x) {
     const double2 pv = p2[t];
     double2 xv = x2[t];
     xv.x = fma(alpha, pv.x, xv.x);
     xv.y = fma(alpha, pv.y, xv.y);
     x2[t] = xv;
   }
+}
+
+__global__ void __launch_bounds__(kThreads) k_x_final(long long n, const double* __restrict__ pb0,
+                                                      const double* __restrict__ pb1, double* __restrict__ x,
+                                                      const PcgState* st) {
+  x_final_body(vblk_self(), n, pb0, pb1, x, st);
 }
 
 void launch_x_final(dd_ctx* c, cudaStream_t s) {
@@ -1690,24 +1696,37 @@ __global__ void __launch_bounds__(kThreads, 8) kb_pcg_init(const BInst* __restri
   pcg_init_body<1>(VBlk{m.y, I.nb_init}, I.g, I.tabS, I.x, bvec(I, b_role), I.r, I.st, I.red, I.cnt + CNT_INIT);
 }
 
+// lag: x += alpha_{k-1} p_{k-1} in this pass (the plain launch's x_lag), else by the x/r update
 template <bool PAIRS>
-__global__ void __launch_bounds__(kThreads, 6) kb_fused_pq(const BInst* __restrict__ B, const int2* __restrict__ vmap) {
+__global__ void __launch_bounds__(kThreads, 6) kb_fused_pq(const BInst* __restrict__ B, const int2* __restrict__ vmap,
+                                                           int lag) {
   const int2 m = vmap[blockIdx.x];
   const BInst& I = B[m.x];
   if (!I.active) return;
+  double* x = lag ? I.x : nullptr;
   if (PAIRS)
-    fused_pq_pairs_body(VBlk{m.y, I.nb_fused}, I.g, I.tabS2, I.z, I.pb0, I.pb1, I.q, nullptr, I.st, I.red,
+    fused_pq_pairs_body(VBlk{m.y, I.nb_fused}, I.g, I.tabS2, I.z, I.pb0, I.pb1, I.q, x, I.st, I.red,
                         I.cnt + CNT_PQ);
   else
-    fused_pq_body<2>(VBlk{m.y, I.nb_fused}, I.g, I.tabS, I.z, I.pb0, I.pb1, I.q, nullptr, I.st, I.red,
+    fused_pq_body<2>(VBlk{m.y, I.nb_fused}, I.g, I.tabS, I.z, I.pb0, I.pb1, I.q, x, I.st, I.red,
                      I.cnt + CNT_PQ);
 }
 
+template <bool UPX>
 __global__ void __launch_bounds__(kThreads) kb_xr_update(const BInst* __restrict__ B, const int2* __restrict__ vmap) {
   const int2 m = vmap[blockIdx.x];
   const BInst& I = B[m.x];
   if (!I.active) return;
-  xr_update_body<true>(VBlk{m.y, I.nb_xr}, I.g.plen, I.pb0, I.pb1, I.q, I.x, I.r, I.st, I.red, I.cnt + CNT_RR);
+  xr_update_body<UPX>(VBlk{m.y, I.nb_xr}, I.g.plen, I.pb0, I.pb1, I.q, I.x, I.r, I.st, I.red, I.cnt + CNT_RR);
+}
+
+// after the running instances' solves, with the lagged x update (two groups at once, 12 instances of
+// 25 to 512 cells, n = 32: the x/r update 17.3 -> 12.8 us, the p update 23.6 -> 24.0)
+__global__ void __launch_bounds__(kThreads) kb_x_final(const BInst* __restrict__ B, const int2* __restrict__ vmap) {
+  const int2 m = vmap[blockIdx.x];
+  const BInst& I = B[m.x];
+  if (!I.active) return;
+  x_final_body(VBlk{m.y, I.nb_vec}, I.g.plen, I.pb0, I.pb1, I.x, I.st);
 }
 
 template <bool ARITH, bool UPD>
@@ -1909,20 +1928,27 @@ void launch_b_pcg_init(const BInst* B, const int2* vmap, int nvb, int b_role, cu
   DD_CUDA(cudaGetLastError());
 }
 
-void launch_b_fused_pq(const BInst* B, const int2* vmap, int nvb, int ypad, bool pairs, cudaStream_t s) {
+void launch_b_fused_pq(const BInst* B, const int2* vmap, int nvb, int ypad, bool pairs, bool lag,
+                       cudaStream_t s) {
   const size_t smem = fused_pq_smem(ypad, pairs);
   static PerDeviceOnce attr;
   once_per_device(attr, [] {
     DD_CUDA(cudaFuncSetAttribute(kb_fused_pq<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     DD_CUDA(cudaFuncSetAttribute(kb_fused_pq<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   });
-  if (pairs) (kb_fused_pq<true><<<nvb, kThreads, smem, s>>>(B, vmap), dd::note_launch());
-  else (kb_fused_pq<false><<<nvb, kThreads, smem, s>>>(B, vmap), dd::note_launch());
+  if (pairs) (kb_fused_pq<true><<<nvb, kThreads, smem, s>>>(B, vmap, lag ? 1 : 0), dd::note_launch());
+  else (kb_fused_pq<false><<<nvb, kThreads, smem, s>>>(B, vmap, lag ? 1 : 0), dd::note_launch());
   DD_CUDA(cudaGetLastError());
 }
 
-void launch_b_xr_update(const BInst* B, const int2* vmap, int nvb, cudaStream_t s) {
-  (kb_xr_update<<<nvb, kThreads, 0, s>>>(B, vmap), dd::note_launch());
+void launch_b_xr_update(const BInst* B, const int2* vmap, int nvb, bool lag, cudaStream_t s) {
+  if (lag) (kb_xr_update<false><<<nvb, kThreads, 0, s>>>(B, vmap), dd::note_launch());
+  else (kb_xr_update<true><<<nvb, kThreads, 0, s>>>(B, vmap), dd::note_launch());
+  DD_CUDA(cudaGetLastError());
+}
+
+void launch_b_x_final(const BInst* B, const int2* vmap, int nvb, cudaStream_t s) {
+  (kb_x_final<<<nvb, kThreads, 0, s>>>(B, vmap), dd::note_launch());
   DD_CUDA(cudaGetLastError());
 }
 
