@@ -28,10 +28,9 @@ namespace dd {
 constexpr int kBandWinMax = 160;
 
 __device__ __forceinline__ double rsqrt_el(double v) { return rsqrt(v); }
-__device__ __forceinline__ float rsqrt_el(float v) { return rsqrtf(v); }
+__device__ __forceinline__ float rsqrt_el(float v) { return rsqrtf(v); }   // wide bands
 
-// T = double, or float for factors whose inverses are rounded to a tensor-core type and for
-// the cell preconditioner (GB300 issues FP32 at 64x the FP64 rate)
+// FP64 (the coarse matrix); FP32 factors take k_band_factor_panel
 template <typename T, int P, int PPT>
 __global__ void __launch_bounds__(1024) k_band_factor_win(T* CB, T* inv, const int* __restrict__ nvec,
                                                           int nmax, int b, int* flag) {
@@ -90,36 +89,21 @@ __global__ void __launch_bounds__(1024) k_band_factor_win(T* CB, T* inv, const i
     for (int u = 0; u < P; ++u) {
       const int k = k0 + u;
       if (k < n) {
-        T il;
-        if constexpr (sizeof(T) == 4) {
-          // FP32: every thread forms the pivot's reciprocal square root itself (identical
-          // values), which saves the barrier that publishing it would take
+        // one thread forms the pivot's reciprocal square root (the FP64 pipe would pay for
+        // every redundant copy)
+        if (t == 0) {
           T piv = win[sk * S];
           if (!(piv > (T)0)) {
-            if (t == 0) atomicOr(flag, 1);
+            atomicOr(flag, 1);
             piv = (T)1;
           }
-          il = rsqrt_el(piv);
-          if (t == 0) {
-            A[(size_t)k * bs] = piv * il;
-            iv[k] = il * il;
-          }
-        } else {
-          // FP64: one thread (the FP64 pipe would pay for every redundant copy)
-          if (t == 0) {
-            T piv = win[sk * S];
-            if (!(piv > (T)0)) {
-              atomicOr(flag, 1);
-              piv = (T)1;
-            }
-            const T l = rsqrt_el(piv);
-            A[(size_t)k * bs] = piv * l;
-            iv[k] = l * l;
-            colk[0] = l;
-          }
-          __syncthreads();
-          il = colk[0];
+          const T l = rsqrt_el(piv);
+          A[(size_t)k * bs] = piv * l;
+          iv[k] = l * l;
+          colk[0] = l;
         }
+        __syncthreads();
+        const T il = colk[0];
         const int dmax = min(b, n - 1 - k);
         for (int d = 1 + t; d <= b; d += blockDim.x) {
           T v = (T)0;
@@ -155,6 +139,144 @@ __global__ void __launch_bounds__(1024) k_band_factor_win(T* CB, T* inv, const i
     }
   }
   cp_async_wait<0>();   // no copy into this block's shared memory outlives it
+}
+
+// FP32 factors of bands up to 160 (the local matrices of the mixed form, whose inverses are rounded
+// to a tensor-core type, and the cell preconditioner): the same window and the same operations in
+// the same order (the same bits), eight columns at a time.  A column's chain (pivot, reciprocal
+// square root, scaling, update of the next column) with two block barriers bounds the rank-1 form at
+// 0.46 us per column whatever the band; here one warp factors a panel of eight columns in its
+// registers (rows over the lanes, Q per lane, the multipliers by shuffle), and the block applies
+// all eight to the trailing window with one read and write of each entry.  The columns that enter
+// are loaded a panel ahead.
+// Order 1209, band 32 (the three local types at L = 2048, n = 32): 549 -> 298 us; order 992, band 63
+// (its cell): 549 -> 330 us.
+constexpr int kPb = 8;
+template <int Q, int PPT>
+__global__ void __launch_bounds__(Q <= 3 ? 512 : 1024) k_band_factor_panel(float* CB, float* inv, const int* __restrict__ nvec,
+                                                            int nmax, int b, int* flag) {
+  extern __shared__ __align__(16) unsigned char fsm_raw[];
+  const int m = blockIdx.x;
+  const int n = nvec[m];
+  const int bs = b + 1, W = b + kPb;
+  const int S = (bs + 1) & ~1;   // as above: even, so that the update's threads fall on different banks
+  const int t = threadIdx.x, T = (int)blockDim.x, lane = t & 31;
+  float* Pn = reinterpret_cast<float*>(fsm_raw);   // L(k + i, k + c) at 8 i + c, i < 32 Q
+  float* win = Pn + 32 * Q * kPb;                  // W columns x S entries, column j in slot j mod W
+  float* A = CB + (size_t)m * nmax * bs;
+  float* iv = inv + (size_t)m * nmax;
+  // this thread's entries (i, j), 0 <= j <= i < b, of the trailing window (behind the panel): linear
+  // index e = i (i + 1) / 2 + j = t, t + T, ...; absent ones are (255, 0), beyond reach
+  unsigned pr[(PPT + 1) / 2];
+#pragma unroll
+  for (int u = 0; u < PPT; ++u) {
+    const int e = t + u * T;
+    int i = 255, j = 0;
+    if (e < b * (b + 1) / 2) {
+      i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);   // first guess, then exact
+      while (i * (i + 1) / 2 > e) --i;
+      while ((i + 2) * (i + 1) / 2 <= e) ++i;
+      j = e - i * (i + 1) / 2;
+    }
+    const unsigned half = ((unsigned)i << 8) | (unsigned)j;
+    if (u & 1) pr[u >> 1] |= half << 16;
+    else pr[u >> 1] = half;
+  }
+  for (int e = t; e < min(W, n) * bs; e += T) win[(e / bs) * S + e % bs] = A[e];
+  __syncthreads();
+  constexpr int kEnter = 4;   // entering values a thread holds: 8 (b + 1) <= 4 T
+  int sk = 0;                 // slot of column k
+  for (int k = 0; k < n; k += kPb) {
+    float en[kEnter];
+#pragma unroll
+    for (int u = 0; u < kEnter; ++u) {
+      const int e = t + u * T, col = k + W + e / bs;
+      en[u] = (e < kPb * bs && col < n) ? __ldcg(A + (size_t)col * bs + e % bs) : 0.0f;
+    }
+    if (t < 32) {
+      float a[kPb][Q];
+#pragma unroll
+      for (int c = 0; c < kPb; ++c) {
+        const int slot = sk + c >= W ? sk + c - W : sk + c;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          const int i = lane + 32 * q, d = i - c;
+          a[c][q] = (d >= 0 && d <= b && k + i < n) ? win[slot * S + d] : 0.0f;
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < kPb; ++c) {
+        float l[Q];
+        if (k + c < n) {   // uniform
+          float piv = __shfl_sync(kFull, a[c][0], c);
+          if (!(piv > 0.0f)) {
+            if (lane == 0) atomicOr(flag, 1);
+            piv = 1.0f;
+          }
+          const float il = rsqrtf(piv);
+          float* out = A + (size_t)(k + c) * bs;
+#pragma unroll
+          for (int q = 0; q < Q; ++q) {
+            const int i = lane + 32 * q, d = i - c;
+            l[q] = d > 0 ? a[c][q] * il : 0.0f;
+            if (d > 0 && d <= b && k + i < n) out[d] = l[q] * il;   // pre-scaled by 1/L(k,k)
+          }
+          if (lane == 0) {
+            out[0] = piv * il;
+            iv[k + c] = il * il;
+          }
+#pragma unroll
+          for (int c2 = c + 1; c2 < kPb; ++c2) {
+            const float l2 = __shfl_sync(kFull, l[0], c2);
+#pragma unroll
+            for (int q = 0; q < Q; ++q) a[c2][q] = fmaf(-l[q], l2, a[c2][q]);
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < Q; ++q) l[q] = 0.0f;
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) Pn[kPb * (lane + 32 * q) + c] = l[q];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < PPT; ++u) {
+      const unsigned half = (u & 1) ? (pr[u >> 1] >> 16) : (pr[u >> 1] & 0xFFFFu);
+      const int i = (int)(half >> 8), j = (int)(half & 0xFFu);
+      if (i < b && k + kPb + i < n) {
+        int slot = sk + kPb + j;
+        if (slot >= W) slot -= W;
+        float* w = win + slot * S + (i - j);
+        const float4* li = reinterpret_cast<const float4*>(Pn + kPb * (kPb + i));
+        const float4* lj = reinterpret_cast<const float4*>(Pn + kPb * (kPb + j));
+        const float4 i0 = li[0], i1 = li[1], j0 = lj[0], j1 = lj[1];
+        float v = *w;
+        v = fmaf(-i0.x, j0.x, v);
+        v = fmaf(-i0.y, j0.y, v);
+        v = fmaf(-i0.z, j0.z, v);
+        v = fmaf(-i0.w, j0.w, v);
+        v = fmaf(-i1.x, j1.x, v);
+        v = fmaf(-i1.y, j1.y, v);
+        v = fmaf(-i1.z, j1.z, v);
+        v = fmaf(-i1.w, j1.w, v);
+        *w = v;
+      }
+    }
+    // the panel's slots take the entering columns
+#pragma unroll
+    for (int u = 0; u < kEnter; ++u) {
+      const int e = t + u * T;
+      if (e < kPb * bs) {
+        int slot = sk + e / bs;
+        if (slot >= W) slot -= W;
+        win[slot * S + e % bs] = en[u];
+      }
+    }
+    __syncthreads();
+    sk += kPb;
+    if (sk >= W) sk -= W;
+  }
 }
 
 // Wide bands (b > 160, the window does not fit in shared memory): blocked right-looking band
@@ -289,7 +411,7 @@ template <typename T>
 static void factor_launch(T* CB, T* RB, T* inv, const int* nvec, int nmat, int nmax, int b, int* flag,
                           cudaStream_t s) {
   if (b <= kBandWinMax) {
-    const size_t smem = sizeof(T) * ((size_t)(b + 1) * (((b + 1) + 1) & ~1) + (size_t)(b + 1) * (1 + 4));
+    size_t smem = sizeof(T) * ((size_t)(b + 1) * (((b + 1) + 1) & ~1) + (size_t)(b + 1) * (1 + 4));
     // PPT triangle pairs per thread, the block at least one thread per entry of a column (the
     // window's entering columns are staged one entry per thread) and at most 1024 threads
     const int tot = b * (b + 1) / 2;
@@ -299,6 +421,25 @@ static void factor_launch(T* CB, T* RB, T* inv, const int* nvec, int nmat, int n
     int threads = ((tot + ppt - 1) / ppt + 31) / 32 * 32;
     threads = std::max(threads, (b + 1 + 31) / 32 * 32);
     threads = std::min(threads, 1024);
+    if constexpr (sizeof(T) == 4) {
+      // one warp factors the panel; the block has a thread for a quarter of the entering values
+      threads = std::min(1024, std::max(threads, (2 * (b + 1) + 31) / 32 * 32));
+#define DD_FPAN(Q_, PPT_)                                                                                          \
+  do {                                                                                                             \
+    static dd::PerDeviceOnce attr;   /* once per device and instance */                                            \
+    once_per_device(attr, [] {                                                                                     \
+      DD_CUDA(cudaFuncSetAttribute(k_band_factor_panel<Q_, PPT_>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
+                                   220 * 1024));                                                                   \
+    });                                                                                                            \
+    smem = sizeof(float) * ((size_t)32 * Q_ * kPb + (size_t)(b + kPb) * ((b + 2) & ~1));                           \
+    (k_band_factor_panel<Q_, PPT_><<<nmat, threads, smem, s>>>(CB, inv, nvec, nmax, b, flag), dd::note_launch());   \
+  } while (0)
+      if (b + kPb <= 64) DD_FPAN(2, 4);         // tot <= 1596
+      else if (ppt == 4) DD_FPAN(3, 4);         // b <= 63
+      else if (b + kPb <= 96) DD_FPAN(3, 8);    // b <= 88: 3916 entries
+      else DD_FPAN(6, 16);
+#undef DD_FPAN
+    } else {
 #define DD_FWIN(PPT_)                                                                                         \
   do {                                                                                                      \
     static dd::PerDeviceOnce attr;   /* once per device and instance */                                     \
@@ -312,6 +453,7 @@ static void factor_launch(T* CB, T* RB, T* inv, const int* nvec, int nmat, int n
     else if (ppt == 8) DD_FWIN(8);
     else DD_FWIN(16);
 #undef DD_FWIN
+    }
   } else {
     const int np = std::min<int>(kPanel, (int)((200 * 1024) / (sizeof(T) * (size_t)(b + 1))));
     if (np < 1) throw Error(DD_EINVAL, "band too wide for the shared-memory panel factorisation");
