@@ -47,7 +47,8 @@ struct TcCfg {
   // went from 6.3 to 5.0 us, the tensor floor of the tile shape.  128 x 256 tiles: one atom,
   // 4 stages (193 KB); 128 x 128 tiles: one atom, 3 stages (97 KB), so that two CTAs share
   // an SM and one's epilogue overlaps the other's MMAs.
-  static constexpr int ATOMS = (BN_ == 160) ? 2 : 1;
+  // 128 x 64 tiles: two atoms, 4 stages (193 KB).
+  static constexpr int ATOMS = (BN_ == 160 || BN_ == 64) ? 2 : 1;
   static constexpr int STAGES = (BN_ == 128 || BN_ == 160) ? 3 : 4;
   // TMEM is allocated in powers of two of at least 32 columns (one FP32 column per output column)
   static constexpr int TMEM_COLS = BN_ <= 32 ? 32 : (BN_ <= 64 ? 64 : (BN_ <= 128 ? 128 : 256));
@@ -624,17 +625,21 @@ __global__ void k_quantize_e4m3(const double* __restrict__ a, long long per_type
     out[t] = to_e4m3(a[t] * scale[t / per_type]);
 }
 
-// Three output-tile shapes, 128 x 256, 128 x 160 and 128 x 128: per output element the K
+// Output-tile shapes 128 x 256, 128 x 160, 128 x 128 and 128 x 64: per output element the K
 // order of the accumulation is the same in all, so the choice changes the speed, not the
 // result.  128 x 160 fits the 2046 interior subdomains of the L = 2048, h = 1/32, delta = 4
-// box in 13 column tiles, so that its 150 tiles make one wave on 152 SMs.
-constexpr int kTileN[3] = {256, 128, 160};
-inline int tile_index(int bn) { return bn == 256 ? 0 : (bn == 128 ? 1 : 2); }
+// box in 13 column tiles, so that its 150 tiles make one wave on 152 SMs.  128 x 64 serves boxes
+// of up to a few hundred subdomains, whose few CTAs are bound by the bytes that each copies for
+// its K loop, most of them columns of R that are not there (37 subdomains, K = 960: 1 MB per CTA
+// with 256 columns, 0.4 MB with 64; 7.2 -> 6.5 us).  Batches choose among the first three.
+constexpr int kTiles = 4, kBatchTiles = 3;
+constexpr int kTileN[kTiles] = {256, 128, 160, 64};
+inline int tile_index(int bn) { return bn == 256 ? 0 : (bn == 128 ? 1 : (bn == 160 ? 2 : 3)); }
 struct GemmPlan {
-  CUtensorMap tA, tB[3];                         // tB[i]: box of kTileN[i] rows of R
-  Tile* tiles[3] = {nullptr, nullptr, nullptr};   // tiles[i]: 128 x kTileN[i] output tiles
-  int ntiles[3] = {0, 0, 0};
-  int cap[3] = {0, 0, 0};
+  CUtensorMap tA, tB[kTiles];                    // tB[i]: box of kTileN[i] rows of R
+  Tile* tiles[kTiles] = {};                       // tiles[i]: 128 x kTileN[i] output tiles
+  int ntiles[kTiles] = {};
+  int cap[kTiles] = {};
   int es = 2;                                     // operand bytes: 1 E4M3, 2 BF16, 4 TF32
 };
 
@@ -654,6 +659,9 @@ static void run_gemm_t(dd_ctx* c, GemmPlan* plan, int bn, const PcgState* st, cu
   else if (bn == 160)
     launch_tc<T, 160>(&plan->tA, tB, plan->tiles[i], plan->ntiles[i], c->kpad, c->kpad, c->kpad, c->Y32, c->kpad,
                       c->dev_err + 8, st, s, ysc, nullptr, pdl);
+  else if (bn == 64)
+    launch_tc<T, 64>(&plan->tA, tB, plan->tiles[i], plan->ntiles[i], c->kpad, c->kpad, c->kpad, c->Y32, c->kpad,
+                     c->dev_err + 8, st, s, ysc, nullptr, pdl);
   else
     launch_tc<T, 128>(&plan->tA, tB, plan->tiles[i], plan->ntiles[i], c->kpad, c->kpad, c->kpad, c->Y32, c->kpad,
                       c->dev_err + 8, st, s, ysc, nullptr, pdl);
@@ -779,7 +787,7 @@ int gemm_setup(dd_ctx* c) {
   const int BK = 128 / es;   // one 128-byte swizzle row of K
   make_tmap(&plan->tA, c->Ainv, es, kpad, (long long)c->ntypes * kpad, BK, 128);
   const int mt = (kpad + 127) / 128;
-  for (int i = 0; i < 3; ++i) {
+  for (int i = 0; i < kTiles; ++i) {
     const int bn = kTileN[i];
     make_tmap(&plan->tB[i], c->Rpack, es, kpad, g.nsub, BK, bn);
     // Tiles in launch order.  Grids of several waves go band by band (per type, one 128-row
@@ -917,10 +925,10 @@ void launch_b_pack(const BInst* B, const int2* vmap, int nvb, int precision, cud
 // order of the accumulation is that of the problem's own launch: results are identical.
 // ----------------------------------------------------------------------------------------
 struct BGemm {
-  CUtensorMap tA, tB[3];
-  Tile* tiles[3] = {nullptr, nullptr, nullptr};
-  const PcgState** tile_st[3] = {nullptr, nullptr, nullptr};
-  int ntiles[3] = {0, 0, 0};
+  CUtensorMap tA, tB[kBatchTiles];
+  Tile* tiles[kBatchTiles] = {};
+  const PcgState** tile_st[kBatchTiles] = {};
+  int ntiles[kBatchTiles] = {};
   int es = 2, kpad = 0, bn = 0;
   float* Y = nullptr;
   int* err = nullptr;
@@ -944,7 +952,7 @@ BGemm* bgemm_create(const std::vector<dd_ctx*>& cs, const std::vector<int>& type
     const int BK = 128 / b->es;
     make_tmap(&b->tA, Ainv_all, b->es, b->kpad, (long long)types * b->kpad, BK, 128);
     const int mt = (b->kpad + 127) / 128;
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < kBatchTiles; ++k) {
       const int bn = kTileN[k];
       make_tmap(&b->tB[k], Rpack_all, b->es, b->kpad, slots, BK, bn);
       std::vector<Tile> tl;
@@ -976,7 +984,7 @@ BGemm* bgemm_create(const std::vector<dd_ctx*>& cs, const std::vector<int>& type
 
 void bgemm_destroy(BGemm* b) {
   if (!b) return;
-  for (int k = 0; k < 3; ++k) {
+  for (int k = 0; k < kBatchTiles; ++k) {
     if (b->tiles[k]) cudaFree(b->tiles[k]);
     if (b->tile_st[k]) cudaFree(b->tile_st[k]);
   }
@@ -1012,7 +1020,8 @@ int bgemm_tune(BGemm* b, cudaStream_t s) {
   float best = 0.0f;
   int best_bn = 256;
   try {
-    for (int bn : kTileN) {
+    for (int k = 0; k < kBatchTiles; ++k) {
+      const int bn = kTileN[k];
       bgemm_run(b, bn, s);
       DD_CUDA(cudaEventRecord(e0, s));
       for (int r = 0; r < 3; ++r) bgemm_run(b, bn, s);
