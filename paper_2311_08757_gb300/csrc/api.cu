@@ -464,7 +464,7 @@ int gmres_run(dd_ctx* c, const double* b, double rtol, int maxit, int* iters, do
     DD_CUDA(cudaMemcpyAsync(c->gm_Vptr, c->gm_V.data(), sizeof(double*) * (m + 1), cudaMemcpyHostToDevice, s));
     DD_CUDA(cudaMemcpyAsync(c->gm_Zptr, c->gm_Z.data(), sizeof(double*) * m, cudaMemcpyHostToDevice, s));
     c->gm_part = (double*)dev_alloc(c, sizeof(double) * (size_t)(m + 1) * 152);
-    c->gm_h = (double*)dev_alloc(c, sizeof(double) * (2 * ld + 1));
+    c->gm_h = (double*)dev_alloc(c, sizeof(double) * (2 * ld + 2));
     c->gm_H = (double*)dev_alloc(c, sizeof(double) * (size_t)ld * m);
     c->gm_cs = (double*)dev_alloc(c, sizeof(double) * m);
     c->gm_sn = (double*)dev_alloc(c, sizeof(double) * m);
@@ -476,7 +476,7 @@ int gmres_run(dd_ctx* c, const double* b, double rtol, int maxit, int* iters, do
     c->gm_alloc = m;
   }
   double* W = c->gm_W;
-  double* nrm2 = c->gm_h + 2 * ld;  // ||w||^2 (the two passes' projections before it)
+  double* nrm2 = c->gm_h + 2 * ld;  // ||w||^2, 1 / ||w|| (the two passes' projections before them)
   auto read_scalar = [&](const double* d) -> double {
     DD_CUDA(cudaMemcpyAsync(c->gm_res_h, d, sizeof(double), cudaMemcpyDeviceToHost, s));
     DD_CUDA(cudaStreamSynchronize(s));
@@ -500,7 +500,7 @@ int gmres_run(dd_ctx* c, const double* b, double rtol, int maxit, int* iters, do
     return DD_OK;
   }
   while (true) {
-    TIMED(KC_XRUPDATE, s, launch_scale_by_norm(c, W, nrm2, c->gm_V[0], s));
+    TIMED(KC_XRUPDATE, s, launch_scale_by_norm(c, W, nrm2, false, c->gm_V[0], s));
     TIMED(KC_MISC, s, launch_gmres_start(c, nrm2, s));
     // Step j: z_j = M^{-1} v_j, w = A z_j orthogonalised against v_0 .. v_j, v_{j+1} = w / ||w||.  The
     // rotation of the Hessenberg column and the residual estimate's copy run on the side stream,
@@ -511,7 +511,7 @@ int gmres_run(dd_ctx* c, const double* b, double rtol, int maxit, int* iters, do
       TIMED(KC_XRUPDATE, s, launch_gm_orthogonalise(c, j, W, nrm2, s));
       DD_CUDA(cudaEventRecord(c->ev_fork, s));
       DD_CUDA(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
-      TIMED(KC_XRUPDATE, s, launch_scale_by_norm(c, W, nrm2, c->gm_V[j + 1], s));
+      TIMED(KC_XRUPDATE, s, launch_scale_by_norm(c, W, nrm2, true, c->gm_V[j + 1], s));
       TIMED(KC_MISC, c->side, launch_givens(c, j, c->gm_res + (j & 1), c->side));
       DD_CUDA(cudaMemcpyAsync(c->gm_res_h + (j & 1), c->gm_res + (j & 1), sizeof(double), cudaMemcpyDeviceToHost,
                               c->side));

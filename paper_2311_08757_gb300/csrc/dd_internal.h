@@ -438,7 +438,7 @@ void launch_adj_dots(dd_ctx* c, const double* u, const double* r, const double* 
 void launch_gm_orthogonalise(dd_ctx* c, int j, double* w, double* nrm2, cudaStream_t s);
 void launch_multiaxpy(dd_ctx* c, int nv, const double* const* V, const double* coef, double sign, double* w,
                       cudaStream_t s);
-void launch_scale_by_norm(dd_ctx* c, const double* w, const double* nrm2, double* v, cudaStream_t s);
+void launch_scale_by_norm(dd_ctx* c, const double* w, const double* nrm2, bool have_inv, double* v, cudaStream_t s);
 void launch_givens(dd_ctx* c, int j, double* res, cudaStream_t s);
 void launch_backsolve(dd_ctx* c, int m, cudaStream_t s);
 void launch_gmres_start(dd_ctx* c, const double* nrm2, cudaStream_t s);

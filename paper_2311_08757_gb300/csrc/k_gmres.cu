@@ -33,7 +33,7 @@ __device__ __forceinline__ double warp_sum_pair(double a, double b) {
 // basis are read from L2 once for both halves of the pass.
 //   MODE 0: out[i] = h_i = (V_i, w)
 //   MODE 1: w -= sum coef_i V_i, then out[i] = (V_i, w) and col[i] = coef_i + out_i
-//   MODE 2: w -= sum coef_i V_i, then nrm2 = out[0] = ||w||^2 and col[nv] = ||w||
+//   MODE 2: w -= sum coef_i V_i, then out[0] = ||w||^2, out[1] = 1 / ||w|| (0 for w = 0), col[nv] = ||w||
 // Bound by the FP64 pipe (2 lanes per clock and SM): 4 n FMAs per basis vector and step over the
 // three passes.  73.8k entries (L = 96, n = 24), average over a cycle of 30: 9.1, 11.3 and 8.5 us for
 // the three modes, of which the FMAs take 8 us in all; the rest is the latency of a block's loads,
@@ -129,7 +129,11 @@ __global__ void __launch_bounds__(kGmThreads) k_gm_pass(long long n, int seg, in
     if (lane == 0 || (lane == 16 && two)) {
       out[e] = a;
       if (MODE == 1) col[e] = cf[e] + a;
-      if (MODE == 2) col[nv] = sqrt(a);
+      if (MODE == 2) {
+        const double nrm = sqrt(a);
+        col[nv] = nrm;
+        out[1] = nrm > 0.0 ? 1.0 / nrm : 0.0;
+      }
     }
   }
   if (threadIdx.x == 0) *counter = 0u;
@@ -146,11 +150,17 @@ __global__ void __launch_bounds__(kThreads) k_multiaxpy(long long n, int nv, con
   }
 }
 
-// v = w / ||w||, the squared norm read from the device
+// v = w / ||w||: nrm2 holds ||w||^2 and, with have_inv, 1 / ||w|| behind it (a square root and a
+// division by every thread took most of the 4.1 us of a pass over 73.8k entries)
 __global__ void __launch_bounds__(kThreads) k_scale_by_norm(long long n, const double* __restrict__ w,
-                                                            const double* __restrict__ nrm2, double* v) {
-  const double nv = sqrt(*nrm2);
-  const double s = nv > 0.0 ? 1.0 / nv : 0.0;
+                                                            const double* __restrict__ nrm2, int have_inv, double* v) {
+  double s;
+  if (have_inv) {
+    s = nrm2[1];
+  } else {
+    const double nv = sqrt(*nrm2);
+    s = nv > 0.0 ? 1.0 / nv : 0.0;
+  }
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x)
     v[t] = w[t] * s;
@@ -225,7 +235,8 @@ __global__ void k_gmres_start(const double* __restrict__ nrm2, double* g, int le
 }
 
 // The two Gram-Schmidt passes of step j on w = W against V_0 .. V_j and the norm of what is left:
-// h and the Hessenberg column j (unrotated, its last entry ||w||) on the device, ||w||^2 in nrm2.
+// h and the Hessenberg column j (unrotated, its last entry ||w||) on the device, ||w||^2 and 1 / ||w|| in
+// nrm2.
 // One block per SM and at least 128 entries each.  L = 96, n = 24, TF32, one GMRES solve of 69
 // steps: 9.2 -> 5.2 ms with the host's read of the estimate one step behind the launches.
 void launch_gm_orthogonalise(dd_ctx* c, int j, double* w, double* nrm2, cudaStream_t s) {
@@ -251,9 +262,9 @@ void launch_multiaxpy(dd_ctx* c, int nv, const double* const* V, const double* c
   DD_CUDA(cudaGetLastError());
 }
 
-void launch_scale_by_norm(dd_ctx* c, const double* w, const double* nrm2, double* v, cudaStream_t s) {
+void launch_scale_by_norm(dd_ctx* c, const double* w, const double* nrm2, bool have_inv, double* v, cudaStream_t s) {
   const long long n = c->g.plen;
-  (k_scale_by_norm<<<grid_blocks(n, kThreads), kThreads, 0, s>>>(n, w, nrm2, v), dd::note_launch());
+  (k_scale_by_norm<<<grid_blocks(n, kThreads), kThreads, 0, s>>>(n, w, nrm2, have_inv ? 1 : 0, v), dd::note_launch());
   DD_CUDA(cudaGetLastError());
 }
 
