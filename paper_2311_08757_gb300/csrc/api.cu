@@ -725,7 +725,7 @@ int dd_setup(const dd_grid* gr, const double* V, size_t nV, void* stream, dd_ctx
     c->z = alloc_vec(c);
     c->pb[0] = alloc_vec(c);
     c->pb[1] = alloc_vec(c);
-    if (g.p == 2) c->p2 = reinterpret_cast<float2*>(alloc_vec(c));   // 8-byte elements, the vectors' layout
+    if (g.p == 2) c->p2 = (float2*)dev_alloc(c, sizeof(float2) * (size_t)(split_p_len(g) + 128)) + 64;   // guarded as the vectors
     c->q = alloc_vec(c);
     c->w1 = alloc_vec(c);
     c->w2 = alloc_vec(c);

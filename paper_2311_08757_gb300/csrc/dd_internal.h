@@ -371,6 +371,7 @@ void launch_check_finite(const double* v, long long n, int* flag, cudaStream_t s
 void launch_pcg_init(dd_ctx* c, const double* b, cudaStream_t s);   // r = b - A x, rr0
 void launch_pupdate(dd_ctx* c, cudaStream_t s);                     // p = z + beta p
 void launch_matvec_pq(dd_ctx* c, cudaStream_t s);                   // q = A p, pq, alpha
+long long split_p_len(const Geo& g);
 void launch_pupdate_pairs(dd_ctx* c, cudaStream_t s);               // p = 2: p update, p also as float pairs
 void launch_matvec_pq_pairs(dd_ctx* c, cudaStream_t s);             // p = 2: q = A p in float pairs, pq, alpha
 void launch_fused_pq(dd_ctx* c, cudaStream_t s);                    // p = z + beta p; q = A p; pq (p = 1)

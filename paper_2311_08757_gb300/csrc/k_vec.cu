@@ -797,6 +797,8 @@ __global__ void __launch_bounds__(kThreads) k_pupdate_pairs(long long n, const d
   double2* pc = reinterpret_cast<double2*>(p_cur(pb0, pb1, k));
   double2* x2 = reinterpret_cast<double2*>(x);
   float4* ps = reinterpret_cast<float4*>(p2);
+  // the element that the last pad slot's corner tap reads (the other form's planes may reach past it)
+  if (blockIdx.x == 0 && threadIdx.x == 0) ps[n / 2] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n / 2;
        t += (long long)gridDim.x * blockDim.x) {
     double2 a = z2[t], b = pp[t];
@@ -814,8 +816,77 @@ __global__ void __launch_bounds__(kThreads) k_pupdate_pairs(long long n, const d
   }
 }
 
+// columns between the two nodes of a pair: half of the cells along x_2
+__host__ __device__ inline int cls_half(const Geo& g) { return g.n * ((g.L + 1) / 2); }
+
+// The same for the register-table matvec: the split p as {hi, hi', lo, lo'} of the nodes in columns a2
+// and a2 + H of a plane (H: half of the cells along x_2), so that its packed operands are two
+// registers of one 16-byte load each.  A plane has H + 2 elements per slot, a2 = -1 .. H: the first
+// and the last repeat the neighbours across the halves and are written but not owned.  Two slots
+// per thread.
+__global__ void __launch_bounds__(kThreads) k_pupdate_pairs_cls(Geo g, int H, unsigned total,
+                                                                const double* __restrict__ z, double* pb0, double* pb1,
+                                                                float4* __restrict__ p4, double* __restrict__ x,
+                                                                const PcgState* st) {
+  pdl_enter();
+  if (st->done) return;
+  const double beta = st->beta;
+  const int k = st->iter;
+  const double alpha = st->alpha;
+  const bool upx = x != nullptr && k > 0;
+  const double* __restrict__ pp = p_prev(pb0, pb1, k);
+  double* __restrict__ pc = p_cur(pb0, pb1, k);
+  const unsigned per = (unsigned)(H + 2) << (g.ylog - 1);   // pairs of slots per plane
+  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+    const unsigned a1 = t / per, e = t - a1 * per;
+    const int a2 = (int)(e >> (g.ylog - 1)) - 1;
+    const long long i0 = (((long long)a1 * g.ncx + a2) << g.ylog) + 2 * (e & (unsigned)(g.Ypad / 2 - 1));
+    const bool own = a2 >= 0 && a2 < H;
+    float2 sp[2][2];
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int col = a2 + b * H;
+      const long long i = i0 + ((long long)(b * H) << g.ylog);
+      const bool in = col >= 0 && col < g.ncx;
+      const double2 zero = make_double2(0.0, 0.0);
+      const double2 zv = in ? *reinterpret_cast<const double2*>(z + i) : zero;
+      double2 v = in ? *reinterpret_cast<const double2*>(pp + i) : zero;
+      if (in && own && upx) {
+        double2 xv = *reinterpret_cast<const double2*>(x + i);
+        xv.x = fma(alpha, v.x, xv.x);
+        xv.y = fma(alpha, v.y, xv.y);
+        *reinterpret_cast<double2*>(x + i) = xv;
+      }
+      v.x = fma(beta, v.x, zv.x);
+      v.y = fma(beta, v.y, zv.y);
+      if (in && own) *reinterpret_cast<double2*>(pc + i) = v;
+      sp[b][0] = f64_split(v.x);
+      sp[b][1] = f64_split(v.y);
+    }
+    float4* out = p4 + 2 * (size_t)t;
+    out[0] = make_float4(sp[0][0].x, sp[1][0].x, sp[0][0].y, sp[1][0].y);
+    out[1] = make_float4(sp[0][1].x, sp[1][1].x, sp[0][1].y, sp[1][1].y);
+  }
+}
+
+bool matvec_cls_shape(const Geo& g, int* CW, int* ncg);
+
+// float2 elements of the split p: the padded vector, or the interleaved planes where those are longer
+long long split_p_len(const Geo& g) {
+  return std::max(g.plen, 2 * ((long long)g.ncx * (cls_half(g) + 2) << g.ylog));
+}
+
 void launch_pupdate_pairs(dd_ctx* c, cudaStream_t s) {
   const long long n = c->g.plen;
+  int CW = 0, ncg = 0;
+  if (c->matvec_tiled && matvec_cls_shape(c->g, &CW, &ncg)) {
+    const int H = cls_half(c->g);
+    const unsigned total = (unsigned)((long long)c->g.ncx * (H + 2) * (c->g.Ypad / 2));   // below 2^31: two per node
+    launch_chain(k_pupdate_pairs_cls, dim3(grid_blocks(total, kThreads)), dim3(kThreads), 0, s, c->pdl != 0, c->g, H,
+                 total, (const double*)c->z, c->pb[0], c->pb[1], reinterpret_cast<float4*>(c->p2), x_lag_target(c),
+                 (const PcgState*)c->st);
+    return;
+  }
   launch_chain(k_pupdate_pairs, dim3(grid_blocks(n / 2, kThreads)), dim3(kThreads), 0, s, c->pdl != 0, n,
                (const double*)c->z, c->pb[0], c->pb[1], c->p2, x_lag_target(c), (const PcgState*)c->st);
 }
@@ -873,18 +944,19 @@ __global__ void __launch_bounds__(kThreads) k_matvec_pq_pairs(Geo g, const float
 // The same pass with the table in registers.  The class of node (a1, a2, slot) depends on a1 and
 // a2 modulo n, so a block takes the planes of one residue r = a1 mod n and, of every cell along x_2,
 // the same W columns: a thread then holds one class for the whole kernel, and its 27 split taps
-// stay in registers.  Per step the block evaluates
-// kClsCells cells of one plane, and every operation of pair_fma works on two of the thread's nodes
-// at once (packed FP32 instructions; the packed two-product negates one factor beforehand, an exact
-// operation).  The split p of the planes a1 - 1 .. a1 + 1 over W + 2 columns is one contiguous run per
-// plane and cell, brought by bulk copies two steps ahead.  Each node's arithmetic is that of k_matvec_pq_pairs, operation by
-// operation (the same q bits); the (p, q) partials are summed in another order.
+// stay in registers.  Per step the block evaluates those columns of kClsPairs pairs of cells of one
+// plane, cell j and the cell half the box further, and every operation of pair_fma works on both
+// nodes at once (packed FP32 instructions; the packed two-product negates one factor beforehand, an
+// exact operation).  The p update stores the split p of such a pair interleaved, so that a tap's packed
+// operands are one 16-byte load.  The planes a1 - 1 .. a1 + 1 over W + 2 columns are one
+// contiguous run per plane and pair, brought by bulk copies two steps ahead.  Each node's arithmetic is
+// that of k_matvec_pq_pairs, operation by operation (the same q bits); the (p, q) partials are
+// summed in another order.
 //
-// L = 64, h = 1/16 (17M padded nodes): 525-590 us with the table slice and p staged through shared
-// memory by the threads (one cell, scalar operations), 375 us with two cells of 256 threads, 345 us
-// with four cells of 128 threads; the FP32 pipe needs 146 us for its 27 x 13 packed operations per
-// two nodes, the copies 134 + 3.4 x 134 MB mostly from L2.  What is left is the moves that pair the
-// operands and the 12 warps an SM holds at 122 registers.
+// L = 64, h = 1/16 (17M padded nodes), per launch in a solve: 232 us with the split p node by node (two
+// 8-byte loads and the moves that pair their halves for every tap of two nodes), 193 us as it is; the
+// FP32 pipe needs 146 us for its 27 x 13 packed operations per two nodes, the copies 134 + 3.4 x 134 MB
+// mostly from L2.  The p update that writes the interleaved form: 94 us against 97.
 constexpr int kClsThreads = 128;
 
 typedef unsigned long long f32x2;
@@ -929,46 +1001,44 @@ __device__ __forceinline__ void pair_fma2(f32x2 t, f32x2 tm, f32x2 xh, f32x2 xl,
   c = fma2(tm, xh, c);
 }
 
-constexpr int kClsStages = 3, kClsCells = 4;
+constexpr int kClsStages = 3, kClsPairs = 2;   // pairs of cells per step
 constexpr int ERR_MATVEC_WAIT = 1 << 9;   // error-word bit: a tile of the matvec did not arrive in time
-// float2 elements of one cell's staged planes, with two zero elements on each side
-__host__ __device__ inline int cls_cell_len(int CW, int Y) { return 3 * (CW + 2) * Y + 4; }
+// float4 elements of one pair's staged planes, with a zero element on each side
+__host__ __device__ inline int cls_cell_len(int CW, int Y) { return 3 * (CW + 2) * Y + 2; }
 
 __global__ void __launch_bounds__(kClsThreads, 3) k_matvec_pq_pairs_cls(Geo g, const float2* __restrict__ tab2,
-                                                                        const float2* __restrict__ p2, double* pb0,
+                                                                        const float4* __restrict__ p4, double* pb0,
                                                                         double* pb1, double* __restrict__ q,
                                                                         PcgState* st, double* partials,
                                                                         unsigned* counter, int CW, int ncg, int* err) {
   pdl_enter();
   if (st->done) return;
-  extern __shared__ __align__(16) float2 smt[];
+  extern __shared__ __align__(16) float4 smt[];
   __shared__ __align__(8) unsigned long long s_bar[kClsStages];
-  const int Y = g.Ypad, yl = g.ylog, n = g.n;
+  const int Y = g.Ypad, yl = g.ylog, n = g.n, H = cls_half(g);
   const int ngrp = n * ncg, gid = (int)blockIdx.x % ngrp, kb = (int)blockIdx.x / ngrp, nbr = (int)gridDim.x / ngrp;
   const int r = gid / ncg, c0 = (gid % ncg) * CW, W = min(CW, n - c0);
   const int row = (W + 2) << yl;                 // one plane's staged run
-  const int cell = cls_cell_len(CW, Y);          // a stage holds kClsCells of them
+  const int cell = cls_cell_len(CW, Y);          // a stage holds kClsPairs of them
   const int cl = (int)threadIdx.x >> yl, slot = (int)threadIdx.x & (Y - 1);
   const bool mine = cl < W;
   const int a1_first = (r == 0) ? n : r;
   const int nplanes = (a1_first <= g.nxi) ? (g.nxi - a1_first) / n + 1 : 0;
-  const int nset = (g.L + kClsCells - 1) / kClsCells;   // sets of kClsCells cells along x_2
+  const int npair = (g.L + 1) / 2, nset = (npair + kClsPairs - 1) / kClsPairs;   // sets of pairs along x_2
   const int nitem = nplanes * nset;
-  const long long c1 = (long long)g.ncx << yl;
+  const long long c1 = (long long)g.ncx << yl, c4 = (long long)(H + 2) << yl;
   const uint32_t bar = smem_u32(s_bar);
   auto fetch = [&](int it, int sl) {             // by one thread: the planes of item it into stage sl
-    const int a1 = a1_first + n * (it / nset), j0 = kClsCells * (it % nset), nc = min(kClsCells, g.L - j0);
-    const uint32_t bytes = (uint32_t)row * sizeof(float2);
+    const int a1 = a1_first + n * (it / nset), j0 = kClsPairs * (it % nset), nc = min(kClsPairs, npair - j0);
+    const uint32_t bytes = (uint32_t)row * sizeof(float4);
     mbar_expect_tx(bar + 8 * sl, 3 * nc * bytes);
     for (int cb = 0; cb < nc; ++cb)
-      for (int pl = 0; pl < 3; ++pl)
-        bulk_g2s(smem_u32(smt + (size_t)(kClsCells * sl + cb) * cell + 2 + pl * row),
-                 p2 + (long long)(a1 - 1 + pl) * c1 + ((long long)(n * (j0 + cb) + c0 - 1) << yl), bytes, bar + 8 * sl);
+      for (int pl = 0; pl < 3; ++pl)   // from column n j + c0 - 1, which is element n j + c0 of the plane
+        bulk_g2s(smem_u32(smt + (size_t)(kClsPairs * sl + cb) * cell + 1 + pl * row),
+                 p4 + (long long)(a1 - 1 + pl) * c4 + ((long long)(n * (j0 + cb) + c0) << yl), bytes, bar + 8 * sl);
   };
-  for (int e = threadIdx.x; e < 4 * kClsCells * kClsStages; e += blockDim.x) {   // the zero elements around each cell
-    const int k = e & 3;
-    smt[(size_t)(e >> 2) * cell + (k < 2 ? k : 3 * row + k)] = make_float2(0.0f, 0.0f);
-  }
+  for (int e = threadIdx.x; e < 2 * kClsPairs * kClsStages; e += blockDim.x)   // the zero elements around each pair
+    smt[(size_t)(e >> 1) * cell + ((e & 1) ? 3 * row + 1 : 0)] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   if (threadIdx.x == 0) {
     for (int i = 0; i < kClsStages; ++i) mbar_init(bar + 8 * i, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1001,36 +1071,39 @@ __global__ void __launch_bounds__(kClsThreads, 3) k_matvec_pq_pairs_cls(Geo g, c
       fetch(it + (kClsStages - 1) * nbr, sl == 0 ? kClsStages - 1 : sl - 1);
     if (!dead && !mbar_wait(bar + 8 * sl, (uint32_t)ph, err, ERR_MATVEC_WAIT)) dead = true;
     if (mine) {
-      const int a1 = a1_first + n * (it / nset), col = kClsCells * n * (it % nset) + c0 + cl;   // in the first cell
-      const long long idx = (long long)a1 * c1 + ((long long)col << yl) + slot, step = (long long)n << yl;
-      bool ok[kClsCells];
-      double pv[kClsCells];
+      const int a1 = a1_first + n * (it / nset), col = kClsPairs * n * (it % nset) + c0 + cl;   // in the first pair
+      const long long idx = (long long)a1 * c1 + ((long long)col << yl) + slot;
+      bool ok[2 * kClsPairs];
+      double pv[2 * kClsPairs];
+      long long at[2 * kClsPairs];
 #pragma unroll
-      for (int b = 0; b < kClsCells; ++b) {
-        ok[b] = col + b * n >= 1 && col + b * n <= g.nxi;
-        pv[b] = ok[b] ? p[idx + b * step] : 0.0;
+      for (int b = 0; b < 2 * kClsPairs; ++b) {
+        const int d = (b >> 1) * n + (b & 1) * H;   // columns past col: pair b / 2, its first or second node
+        ok[b] = col + (b >> 1) * n < H && col + d >= 1 && col + d <= g.nxi;
+        at[b] = idx + ((long long)d << yl);
+        pv[b] = ok[b] ? p[at[b]] : 0.0;
       }
-      const float2* x = smt + (size_t)(kClsCells * sl) * cell + 2 + row + ((cl + 1) << yl) + slot;   // plane a1, this column
-      f32x2 hs[kClsCells / 2], ls[kClsCells / 2];
+      const float4* x = smt + (size_t)(kClsPairs * sl) * cell + 1 + row + ((cl + 1) << yl) + slot;   // plane a1, this column
+      f32x2 hs[kClsPairs], ls[kClsPairs];
 #pragma unroll
-      for (int b = 0; b < kClsCells / 2; ++b) hs[b] = ls[b] = 0;
+      for (int b = 0; b < kClsPairs; ++b) hs[b] = ls[b] = 0;
 #pragma unroll
       for (int tap = 0; tap < 27; ++tap) {
-        const float2* xt = x + (tap / 9 - 1) * row + ((tap / 3) % 3 - 1) * Y + tap % 3 - 1;
+        const float4* xt = x + (tap / 9 - 1) * row + ((tap / 3) % 3 - 1) * Y + tap % 3 - 1;
 #pragma unroll
-        for (int b = 0; b < kClsCells / 2; ++b) {
-          const float2 va = xt[2 * b * cell], vb = xt[(2 * b + 1) * cell];
-          pair_fma2(th[tap], tl[tap], pack2(va.x, vb.x), pack2(va.y, vb.y), hs[b], ls[b]);
+        for (int b = 0; b < kClsPairs; ++b) {
+          const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(xt + b * cell);
+          pair_fma2(th[tap], tl[tap], v.x, v.y, hs[b], ls[b]);
         }
       }
 #pragma unroll
-      for (int b = 0; b < kClsCells; ++b) {
+      for (int b = 0; b < 2 * kClsPairs; ++b) {
         float h2[2], l2[2];
         unpack2(hs[b / 2], h2[0], h2[1]);
         unpack2(ls[b / 2], l2[0], l2[1]);
         if (ok[b]) {
           const double qv = f32_to_f64(h2[b & 1]) + f32_to_f64(l2[b & 1]);
-          q[idx + b * step] = qv;
+          q[at[b]] = qv;
           acc[0] = fma(pv[b], qv, acc[0]);
         }
       }
@@ -1070,17 +1143,17 @@ void launch_matvec_pq_pairs(dd_ctx* c, cudaStream_t s) {
   int CW = 0, ncg = 0;
   if (c->matvec_tiled && matvec_cls_shape(g, &CW, &ncg)) {
     const int threads = (CW * g.Ypad + 31) / 32 * 32;
-    const size_t smem = sizeof(float2) * kClsStages * kClsCells * (size_t)cls_cell_len(CW, g.Ypad);
+    const size_t smem = sizeof(float4) * kClsStages * kClsPairs * (size_t)cls_cell_len(CW, g.Ypad);
     static PerDeviceOnce attr;
     once_per_device(attr, [] {
       DD_CUDA(cudaFuncSetAttribute(k_matvec_pq_pairs_cls, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     });
     int per_sm = 0;
     DD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_matvec_pq_pairs_cls, threads, smem));
-    const int groups = g.n * ncg, items = g.L * ((g.L + kClsCells - 1) / kClsCells);
+    const int groups = g.n * ncg, items = g.L * (((g.L + 1) / 2 + kClsPairs - 1) / kClsPairs);
     const int nbr = std::max(1, std::min({152 * std::max(per_sm, 1) / groups, items, kMaxRedBlocks / groups}));
     launch_chain(k_matvec_pq_pairs_cls, dim3(groups * nbr), dim3(threads), smem, s, c->pdl != 0, g,
-                 (const float2*)c->tabS2, (const float2*)c->p2, c->pb[0], c->pb[1], c->q, c->st, c->red,
+                 (const float2*)c->tabS2, (const float4*)c->p2, c->pb[0], c->pb[1], c->q, c->st, c->red,
                  c->cnt + CNT_PQ, CW, ncg, c->dev_err + 8);
     return;
   }
