@@ -402,11 +402,10 @@ int dd_coarse_matrix(dd_ctx* ctx, double* A0_host);
  *                       on the node columns it owns, updates x (unless DD_OPT_X_LAG) and sums
  *                       (r, r) and takes the stop test), and the prolong-sum stores r - alpha q;
  *                       one kernel fewer per iteration.  x and r take the same values as with
- *                       0; (r, r) is summed in another order.  On the L = 2048, h = 1/32 box a
- *                       PCG iteration took 104.5 us against 99.3 us with 0 (106.0 us without
- *                       DD_OPT_X_LAG): the packing blocks, one per overlapping subdomain, form
- *                       r - alpha q and (r, r) slower than the separate update does, so off by
- *                       default; -1: off [0]
+ *                       0; (r, r) is summed in another order.  0: off; -1: on for at most 512
+ *                       subdomains, where the launch saved counts for more (L = 37, h = 1/32:
+ *                       39.5 -> 37.9 us per PCG iteration) than the columns that two packing
+ *                       blocks both form (L = 2048: 95.7 -> 100.8 us) [-1]
  *   DD_OPT_TILED3       p = 2 with float pairs: 1 evaluates q = A_sigma p with the split table in
  *                       registers (each block takes the planes of one residue a1 mod n and the
  *                       same columns of every cell, so a thread keeps one class) and the split p

@@ -357,6 +357,15 @@ bool fuse_xr_possible(const dd_ctx* c) {
          c->fused_pq_opt != 0 && c->g.nsub <= kMaxRedBlocksHost;
 }
 
+// Without the option, boxes of up to 512 subdomains take the fused form: a launch less per iteration
+// counts for more there than the columns that two subdomains both read and update.  Per iteration, BF16,
+// n = 32: L = 37 39.5 -> 37.9 us, L = 256 43.0 -> 40.6, L = 512 49.5 -> 48.0, but L = 1024 64.9 -> 65.5 and
+// L = 2048 95.7 -> 100.8 us; n = 12: L = 37 30.8 -> 28.5, L = 512 35.1 -> 33.8, L = 1024 39.6 -> 40.2 us.
+constexpr int kFuseXrMaxSub = 512;
+bool fuse_xr(const dd_ctx* c) {
+  return c->fuse_xr || (c->fuse_xr_opt < 0 && fuse_xr_possible(c) && c->g.nsub <= kFuseXrMaxSub);
+}
+
 void pcg_iteration(dd_ctx* c) {
   cudaStream_t s = c->stream;
   if (c->g.p == 1 && c->fused_pq_opt != 0) {   // fused, two nodes per thread unless option 1
@@ -368,7 +377,7 @@ void pcg_iteration(dd_ctx* c) {
     TIMED(KC_PUPDATE, s, launch_pupdate(c, s));
     TIMED(KC_STENCIL, s, launch_matvec_pq(c, s));
   }
-  if (c->fuse_xr) {
+  if (fuse_xr(c)) {
     TIMED(KC_PACK_XR, s, launch_pack_xr(c, s));
     precond(c, c->r, 2, nullptr, true);
   } else {

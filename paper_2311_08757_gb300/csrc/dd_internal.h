@@ -173,12 +173,12 @@ struct dd_ctx {
   int prolong_tables_opt = 1;       // 0: owners in closed form where it holds (slower: 28.1 against 24.5 us at L = 2048)
   int4 ptypes = {0, 0, 0, 0};       // p = 1: type ids of the left end, interior and right end subdomains
   int pdl = 0;                      // PCG chain kernels launched with programmatic dependent launch
-  int fuse_xr_opt = 0;              // x/r update fused into the packing: 1 on, 0 or -1 off
+  int fuse_xr_opt = -1;             // x/r update fused into the packing: 1 on, 0 off, -1 by the number of subdomains
   int matvec_tiled = 1;             // p = 2 float pairs: the register-table matvec where it fits
   // x_{k+1} = x_k + alpha_k p_k deferred to iteration k + 1's p update, which reads p_k anyway,
   // and one final update after the last iteration: the x/r update then streams r and q only
   int x_lag = 1;
-  int fuse_xr = 0;                  // the resolved choice
+  int fuse_xr = 0;                  // asked for (option 1; a batch fuses in that case only)
   int pq_pairs_opt = -1;            // q = A_sigma p of the fused p = 1 kernel: -1 automatic, 0 FP64, 1 float pairs
   int pq_pairs = 0;                 // the resolved choice
   dd::Timer timer;
