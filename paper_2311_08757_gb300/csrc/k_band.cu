@@ -185,13 +185,19 @@ __global__ void __launch_bounds__(Q <= 3 ? 512 : 1024) k_band_factor_panel(float
   for (int e = t; e < min(W, n) * bs; e += T) win[(e / bs) * S + e % bs] = A[e];
   __syncthreads();
   constexpr int kEnter = 4;   // entering values a thread holds: 8 (b + 1) <= 4 T
+  int ec[kEnter], ed[kEnter];   // their columns in the panel (8: none) and places in the column
+#pragma unroll
+  for (int u = 0; u < kEnter; ++u) {
+    ec[u] = min((t + u * T) / bs, kPb);
+    ed[u] = (t + u * T) % bs;
+  }
   int sk = 0;                 // slot of column k
   for (int k = 0; k < n; k += kPb) {
     float en[kEnter];
 #pragma unroll
     for (int u = 0; u < kEnter; ++u) {
-      const int e = t + u * T, col = k + W + e / bs;
-      en[u] = (e < kPb * bs && col < n) ? __ldcg(A + (size_t)col * bs + e % bs) : 0.0f;
+      const int col = k + W + ec[u];
+      en[u] = (ec[u] < kPb && col < n) ? __ldcg(A + (size_t)col * bs + ed[u]) : 0.0f;
     }
     if (t < 32) {
       float a[kPb][Q];
@@ -240,37 +246,46 @@ __global__ void __launch_bounds__(Q <= 3 ? 512 : 1024) k_band_factor_panel(float
       }
     }
     __syncthreads();
+    // all entries of four pairs are loaded before the first is stored back
+    constexpr int G = PPT < 4 ? PPT : 4;
 #pragma unroll
-    for (int u = 0; u < PPT; ++u) {
-      const unsigned half = (u & 1) ? (pr[u >> 1] >> 16) : (pr[u >> 1] & 0xFFFFu);
-      const int i = (int)(half >> 8), j = (int)(half & 0xFFu);
-      if (i < b && k + kPb + i < n) {
-        int slot = sk + kPb + j;
-        if (slot >= W) slot -= W;
-        float* w = win + slot * S + (i - j);
-        const float4* li = reinterpret_cast<const float4*>(Pn + kPb * (kPb + i));
-        const float4* lj = reinterpret_cast<const float4*>(Pn + kPb * (kPb + j));
-        const float4 i0 = li[0], i1 = li[1], j0 = lj[0], j1 = lj[1];
-        float v = *w;
-        v = fmaf(-i0.x, j0.x, v);
-        v = fmaf(-i0.y, j0.y, v);
-        v = fmaf(-i0.z, j0.z, v);
-        v = fmaf(-i0.w, j0.w, v);
-        v = fmaf(-i1.x, j1.x, v);
-        v = fmaf(-i1.y, j1.y, v);
-        v = fmaf(-i1.z, j1.z, v);
-        v = fmaf(-i1.w, j1.w, v);
-        *w = v;
+    for (int u0 = 0; u0 < PPT; u0 += G) {
+      float v[G];
+      float* w[G];
+#pragma unroll
+      for (int u = u0; u < u0 + G; ++u) {
+        const unsigned half = (u & 1) ? (pr[u >> 1] >> 16) : (pr[u >> 1] & 0xFFFFu);
+        const int i = (int)(half >> 8), j = (int)(half & 0xFFu);
+        w[u - u0] = nullptr;
+        if (i < b && k + kPb + i < n) {
+          int slot = sk + kPb + j;
+          if (slot >= W) slot -= W;
+          w[u - u0] = win + slot * S + (i - j);
+          const float4* li = reinterpret_cast<const float4*>(Pn + kPb * (kPb + i));
+          const float4* lj = reinterpret_cast<const float4*>(Pn + kPb * (kPb + j));
+          const float4 i0 = li[0], i1 = li[1], j0 = lj[0], j1 = lj[1];
+          float x = *w[u - u0];
+          x = fmaf(-i0.x, j0.x, x);
+          x = fmaf(-i0.y, j0.y, x);
+          x = fmaf(-i0.z, j0.z, x);
+          x = fmaf(-i0.w, j0.w, x);
+          x = fmaf(-i1.x, j1.x, x);
+          x = fmaf(-i1.y, j1.y, x);
+          x = fmaf(-i1.z, j1.z, x);
+          v[u - u0] = fmaf(-i1.w, j1.w, x);
+        }
       }
+#pragma unroll
+      for (int u = 0; u < G; ++u)
+        if (w[u] != nullptr) *w[u] = v[u];
     }
     // the panel's slots take the entering columns
 #pragma unroll
     for (int u = 0; u < kEnter; ++u) {
-      const int e = t + u * T;
-      if (e < kPb * bs) {
-        int slot = sk + e / bs;
+      if (ec[u] < kPb) {
+        int slot = sk + ec[u];
         if (slot >= W) slot -= W;
-        win[slot * S + e % bs] = en[u];
+        win[slot * S + ed[u]] = en[u];
       }
     }
     __syncthreads();
