@@ -469,7 +469,13 @@ constexpr int kFusedCols = 32;
 // U2 = 2: each thread evaluates two nodes (e, e + blockDim) per pass, their 9-tap chains
 // interleaved; the (p, q) partial is accumulated in the same node order as with U2 = 1, so the
 // result is bit-identical.
-template <int U2>
+//
+// LAT (both forms below): for grids of few blocks per SM, where nothing hides a thread's round trips to
+// L2.  A thread's staged nodes are all loaded before the first is stored (five passes of 256
+// threads at Ypad = 32 were five round trips), and the table of a pass is loaded during the one
+// before, that of the first pass before the staging.  The same operations in the same order; it
+// takes two to three times the registers, which costs more than it gives once blocks queue.
+template <int U2, bool LAT>
 __device__ __forceinline__ void fused_pq_body(VBlk vb, Geo g, const double* __restrict__ tab,
                                               const double* __restrict__ z, double* pb0, double* pb1,
                                               double* __restrict__ q, double* __restrict__ x, PcgState* st,
@@ -497,13 +503,35 @@ __device__ __forceinline__ void fused_pq_body(VBlk vb, Geo g, const double* __re
     const long long gbase = (long long)(a0 - 1) << yl;
     __syncthreads();
     const int nown = own << yl;
-    for (int e = threadIdx.x; e < nload; e += blockDim.x) {
+    double tc[2][9];
+    auto load_table = [&](int e, double (&t)[2][9]) {   // of nodes e and e + blockDim.x
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const int f = e + b * (int)blockDim.x < nown ? e + b * (int)blockDim.x : min(e, nown - 1);
+        const int cls = ((a0 + (f >> yl)) % g.n) * Y + (f & (Y - 1));
+#pragma unroll
+        for (int k = 0; k < 9; ++k) t[b][k] = __ldg(tab + (size_t)k * g.ncls + cls);
+      }
+    };
+    if (LAT) load_table(threadIdx.x, tc);
+    constexpr int SU = LAT ? 5 : 1;
+    for (int e0 = threadIdx.x; e0 < nload; e0 += SU * blockDim.x) {
       // x is loaded beside p_{k-1} and z (one memory round trip per pass), stored for own nodes
-      const bool mine = upx && e >= Y && e < Y + nown;
-      const double pv = pp[gbase + e], zv = z[gbase + e];
-      const double xv = mine ? x[gbase + e] : 0.0;
-      sp[e] = fma(beta, pv, zv);
-      if (mine) x[gbase + e] = fma(alpha, pv, xv);
+      double pv[SU], zv[SU], xv[SU];
+#pragma unroll
+      for (int u = 0; u < SU; ++u) {
+        const int e = e0 + u * (int)blockDim.x;
+        const bool in = SU == 1 || e < nload;
+        pv[u] = in ? pp[gbase + e] : 0.0;
+        zv[u] = in ? z[gbase + e] : 0.0;
+        xv[u] = (upx && e >= Y && e < Y + nown) ? x[gbase + e] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < SU; ++u) {
+        const int e = e0 + u * (int)blockDim.x;
+        if (SU == 1 || e < nload) sp[e] = fma(beta, pv[u], zv[u]);
+        if (upx && e >= Y && e < Y + nown) x[gbase + e] = fma(alpha, pv[u], xv[u]);
+      }
     }
     if (threadIdx.x == 0) sp[nload] = 0.0;   // corner tap of the last (pad) slot of a partial tile
     __syncthreads();
@@ -531,17 +559,35 @@ __device__ __forceinline__ void fused_pq_body(VBlk vb, Geo g, const double* __re
         const int f = two ? e1 : e;   // a valid node for the masked second chain
         const int se0 = e + Y, se1 = f + Y;
         const double pv0 = sp[se0], pv1 = sp[se1];
-        const int cls0 = ((a0 + (e >> yl)) % g.n) * Y + (e & (Y - 1));
-        const int cls1 = ((a0 + (f >> yl)) % g.n) * Y + (f & (Y - 1));
         double q0 = 0.0, q1 = 0.0;
+        if (LAT) {
+          double tn[2][9];
+          const int en = e + 2 * (int)blockDim.x;
+          if (en < nown) load_table(en, tn);
 #pragma unroll
-        for (int dx = -1; dx <= 1; ++dx)
-#pragma unroll
-          for (int dy = -1; dy <= 1; ++dy) {
-            const double* tt = tab + (size_t)((dx + 1) * 3 + (dy + 1)) * g.ncls;
-            q0 = fma(__ldg(tt + cls0), sp[se0 + dx * Y + dy], q0);
-            q1 = fma(__ldg(tt + cls1), sp[se1 + dx * Y + dy], q1);
+          for (int k = 0; k < 9; ++k) {
+            const int o = (k / 3 - 1) * Y + k % 3 - 1;
+            q0 = fma(tc[0][k], sp[se0 + o], q0);
+            q1 = fma(tc[1][k], sp[se1 + o], q1);
           }
+          if (en < nown)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+              tc[0][k] = tn[0][k];
+              tc[1][k] = tn[1][k];
+            }
+        } else {
+          const int cls0 = ((a0 + (e >> yl)) % g.n) * Y + (e & (Y - 1));
+          const int cls1 = ((a0 + (f >> yl)) % g.n) * Y + (f & (Y - 1));
+#pragma unroll
+          for (int dx = -1; dx <= 1; ++dx)
+#pragma unroll
+            for (int dy = -1; dy <= 1; ++dy) {
+              const double* tt = tab + (size_t)((dx + 1) * 3 + (dy + 1)) * g.ncls;
+              q0 = fma(__ldg(tt + cls0), sp[se0 + dx * Y + dy], q0);
+              q1 = fma(__ldg(tt + cls1), sp[se1 + dx * Y + dy], q1);
+            }
+        }
         pc[gbase + se0] = pv0;
         q[gbase + se0] = q0;
         acc[0] = fma(pv0, q0, acc[0]);
@@ -574,19 +620,17 @@ __device__ __forceinline__ void fused_pq_body(VBlk vb, Geo g, const double* __re
 // instructions per node (p update, q = hi + lo, the partial) instead of eleven.  The split table is class-major (a
 // class's taps are five 16-byte loads), p_k is written back from the staging loop, and each
 // thread evaluates two nodes (e, e + blockDim) per pass with their chains interleaved.
-__device__ __forceinline__ void pair_taps(const float2* __restrict__ tab2, int cls, const float2* x, int Y,
-                                          float& hs, float& ls) {
+__device__ __forceinline__ void pair_table(const float2* __restrict__ tab2, int cls, float (&t)[18]) {
   const float4* tr = reinterpret_cast<const float4*>(tab2 + (size_t)cls * kPairTapStride);
-  float t[18];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const float4 v = __ldg(tr + k);
     t[4 * k] = v.x; t[4 * k + 1] = v.y; t[4 * k + 2] = v.z; t[4 * k + 3] = v.w;
   }
-  {
-    const float4 v = __ldg(tr + 4);
-    t[16] = v.x; t[17] = v.y;
-  }
+  const float4 v = __ldg(tr + 4);
+  t[16] = v.x; t[17] = v.y;
+}
+__device__ __forceinline__ void pair_taps(const float (&t)[18], const float2* x, int Y, float& hs, float& ls) {
 #pragma unroll
   for (int dx = -1; dx <= 1; ++dx)
 #pragma unroll
@@ -597,6 +641,7 @@ __device__ __forceinline__ void pair_taps(const float2* __restrict__ tab2, int c
     }
 }
 
+template <bool LAT>
 __device__ __forceinline__ void fused_pq_pairs_body(VBlk vb, Geo g, const float2* __restrict__ tab2,
                                                     const double* __restrict__ z, double* pb0, double* pb1,
                                                     double* __restrict__ q, double* __restrict__ x, PcgState* st,
@@ -628,33 +673,74 @@ __device__ __forceinline__ void fused_pq_pairs_body(VBlk vb, Geo g, const float2
     const int nown = own << yl;
     const long long gbase = (long long)(a0 - 1) << yl;
     __syncthreads();
-    for (int e = threadIdx.x; e < nload; e += blockDim.x) {
-      // x is loaded beside p_{k-1} and z (one memory round trip per pass), stored for own nodes
-      const bool own_e = e >= Y && e < Y + nown;
-      const double pprev = pp[gbase + e], zv = z[gbase + e];
-      const double xv = (upx && own_e) ? x[gbase + e] : 0.0;
-      const double pv = fma(beta, pprev, zv);
-      sp2[e] = f64_split(pv);
-      if (own_e) {
-        pc[gbase + e] = pv;
-        spd[e - Y] = pv;
-        if (upx) x[gbase + e] = fma(alpha, pprev, xv);
-      }
-    }
-    if (threadIdx.x == 0) sp2[nload] = make_float2(0.0f, 0.0f);   // corner tap of the last pad slot
-    __syncthreads();
     // class column (a0 + e / Y) mod n, advanced by cstep columns per pass
     int cm = (a0 + (threadIdx.x >> yl)) % g.n;
     int cm1 = cm + cstep;
     while (cm1 >= g.n) cm1 -= g.n;
+    const int slot = threadIdx.x & (Y - 1);   // blockDim is a multiple of Y
+    float t0[18], t1[18];
+    if (LAT) {
+      pair_table(tab2, cm * Y + slot, t0);
+      pair_table(tab2, cm1 * Y + slot, t1);
+    }
+    constexpr int SU = LAT ? 5 : 1;
+    for (int e0 = threadIdx.x; e0 < nload; e0 += SU * blockDim.x) {
+      // x is loaded beside p_{k-1} and z (one memory round trip per pass), stored for own nodes
+      double pprev[SU], zv[SU], xv[SU];
+#pragma unroll
+      for (int u = 0; u < SU; ++u) {
+        const int e = e0 + u * (int)blockDim.x;
+        const bool in = SU == 1 || e < nload;
+        pprev[u] = in ? pp[gbase + e] : 0.0;
+        zv[u] = in ? z[gbase + e] : 0.0;
+        xv[u] = (upx && e >= Y && e < Y + nown) ? x[gbase + e] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < SU; ++u) {
+        const int e = e0 + u * (int)blockDim.x;
+        if (SU > 1 && e >= nload) break;
+        const double pv = fma(beta, pprev[u], zv[u]);
+        sp2[e] = f64_split(pv);
+        if (e >= Y && e < Y + nown) {
+          pc[gbase + e] = pv;
+          spd[e - Y] = pv;
+          if (upx) x[gbase + e] = fma(alpha, pprev[u], xv[u]);
+        }
+      }
+    }
+    if (threadIdx.x == 0) sp2[nload] = make_float2(0.0f, 0.0f);   // corner tap of the last pad slot
+    __syncthreads();
     for (int e = threadIdx.x; e < nown; e += 2 * blockDim.x) {
       const int e1 = e + blockDim.x;
       const bool two = e1 < nown;
       const int f = two ? e1 : e;   // a valid node for the masked second chain
-      const int slot = e & (Y - 1);
       float h0 = 0.0f, l0 = 0.0f, h1 = 0.0f, l1 = 0.0f;
-      pair_taps(tab2, cm * Y + slot, sp2 + e + Y, Y, h0, l0);
-      pair_taps(tab2, cm1 * Y + slot, sp2 + f + Y, Y, h1, l1);
+      if (!LAT) {
+        pair_table(tab2, cm * Y + slot, t0);
+        pair_taps(t0, sp2 + e + Y, Y, h0, l0);
+        pair_table(tab2, cm1 * Y + slot, t1);
+        pair_taps(t1, sp2 + f + Y, Y, h1, l1);
+      }
+      cm += 2 * cstep;
+      while (cm >= g.n) cm -= g.n;
+      cm1 += 2 * cstep;
+      while (cm1 >= g.n) cm1 -= g.n;
+      if (LAT) {
+        float n0[18], n1[18];
+        const bool more = e + 2 * (int)blockDim.x < nown;
+        if (more) {
+          pair_table(tab2, cm * Y + slot, n0);
+          pair_table(tab2, cm1 * Y + slot, n1);
+        }
+        pair_taps(t0, sp2 + e + Y, Y, h0, l0);
+        pair_taps(t1, sp2 + f + Y, Y, h1, l1);
+        if (more)
+#pragma unroll
+          for (int k = 0; k < 18; ++k) {
+            t0[k] = n0[k];
+            t1[k] = n1[k];
+          }
+      }
       const double q0 = f32_to_f64(h0) + f32_to_f64(l0);
       q[gbase + Y + e] = q0;
       acc[0] = fma(spd[e], q0, acc[0]);
@@ -663,10 +749,6 @@ __device__ __forceinline__ void fused_pq_pairs_body(VBlk vb, Geo g, const float2
         q[gbase + Y + e1] = q1;
         acc[0] = fma(spd[e1], q1, acc[0]);
       }
-      cm += 2 * cstep;
-      while (cm >= g.n) cm -= g.n;
-      cm1 += 2 * cstep;
-      while (cm1 >= g.n) cm1 -= g.n;
     }
   }
   double tot[1];
@@ -682,12 +764,13 @@ __device__ __forceinline__ void fused_pq_pairs_body(VBlk vb, Geo g, const float2
   }
 }
 
+template <bool LAT>
 __global__ void __launch_bounds__(kThreads) k_fused_pq_pairs(Geo g, const float2* __restrict__ tab2,
                                                              const double* __restrict__ z, double* pb0, double* pb1,
                                                              double* __restrict__ q, double* __restrict__ x,
                                                              PcgState* st, double* partials, unsigned* counter) {
   pdl_enter();
-  fused_pq_pairs_body(vblk_self(), g, tab2, z, pb0, pb1, q, x, st, partials, counter);
+  fused_pq_pairs_body<LAT>(vblk_self(), g, tab2, z, pb0, pb1, q, x, st, partials, counter);
 }
 
 static size_t fused_pq_smem(int ypad, bool pairs) {
@@ -695,14 +778,20 @@ static size_t fused_pq_smem(int ypad, bool pairs) {
   return pairs ? n * sizeof(float2) + (size_t)kFusedCols * ypad * sizeof(double) : n * sizeof(double);
 }
 
-template <int U2>
+template <int U2, bool LAT>
 __global__ void __launch_bounds__(kThreads) k_fused_pq(Geo g, const double* __restrict__ tab,
                                                        const double* __restrict__ z, double* pb0, double* pb1,
                                                        double* __restrict__ q, double* __restrict__ x, PcgState* st,
                                                        double* partials, unsigned* counter) {
   pdl_enter();
-  fused_pq_body<U2>(vblk_self(), g, tab, z, pb0, pb1, q, x, st, partials, counter);
+  fused_pq_body<U2, LAT>(vblk_self(), g, tab, z, pb0, pb1, q, x, st, partials, counter);
 }
+
+// LAT up to one tile per SM at Ypad = 32, in proportion to the staged nodes of a thread otherwise.
+// Per PCG iteration, BF16, without and with it: n = 32, L = 37 37.8 / 36.9 us, L = 256 42.1 / 42.0, L = 400
+// 45.0 / 51.1; Ypad = 64 (n = 32, l = 1.5) L = 37 51.0 / 48.4, L = 304 61.4 / 58.0, L = 400 70.4 / 74.6; n = 16
+// the same up to L = 304.  FP64 local solves: n = 32, L = 128 90.9 / 89.6, L = 400 160.0 / 166.5.
+static bool fused_lat(const Geo& g, int ntiles) { return ntiles * kFusedCols <= 152 * g.Ypad; }
 
 void launch_fused_pq(dd_ctx* c, cudaStream_t s) {
   const Geo& g = c->g;
@@ -711,21 +800,25 @@ void launch_fused_pq(dd_ctx* c, cudaStream_t s) {
   const size_t smem = fused_pq_smem(g.Ypad, c->pq_pairs != 0);
   static PerDeviceOnce attr;   // once per device
   once_per_device(attr, [] {
-    DD_CUDA(cudaFuncSetAttribute(k_fused_pq<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    DD_CUDA(cudaFuncSetAttribute(k_fused_pq<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    DD_CUDA(cudaFuncSetAttribute(k_fused_pq_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    const auto big = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    DD_CUDA(cudaFuncSetAttribute(k_fused_pq<1, false>, big, 200 * 1024));
+    DD_CUDA(cudaFuncSetAttribute(k_fused_pq<2, false>, big, 200 * 1024));
+    DD_CUDA(cudaFuncSetAttribute(k_fused_pq<2, true>, big, 200 * 1024));
+    DD_CUDA(cudaFuncSetAttribute(k_fused_pq_pairs<false>, big, 200 * 1024));
+    DD_CUDA(cudaFuncSetAttribute(k_fused_pq_pairs<true>, big, 200 * 1024));
   });
-  const bool pdl = c->pdl != 0;
+  const bool pdl = c->pdl != 0, lat = fused_lat(g, ntiles);
   if (c->pq_pairs) {
-    launch_chain(k_fused_pq_pairs, dim3(nb), dim3(kThreads), smem, s, pdl, g, (const float2*)c->tabS2,
-                 (const double*)c->z, c->pb[0], c->pb[1], c->q, x_lag_target(c), c->st, c->red, c->cnt + CNT_PQ);
+    launch_chain(lat ? k_fused_pq_pairs<true> : k_fused_pq_pairs<false>, dim3(nb), dim3(kThreads), smem, s, pdl, g,
+                 (const float2*)c->tabS2, (const double*)c->z, c->pb[0], c->pb[1], c->q, x_lag_target(c), c->st, c->red,
+                 c->cnt + CNT_PQ);
     return;
   }
   // two nodes per thread and pass by default: 53.0 against 53.8 us per launch on the
   // L = 2048, h = 1/32 box, the same bits
-  launch_chain(c->fused_pq_opt != 1 ? k_fused_pq<2> : k_fused_pq<1>, dim3(nb), dim3(kThreads), smem, s, pdl, g,
-               (const double*)c->tabS, (const double*)c->z, c->pb[0], c->pb[1], c->q, x_lag_target(c), c->st,
-               c->red, c->cnt + CNT_PQ);
+  launch_chain(c->fused_pq_opt == 1 ? k_fused_pq<1, false> : (lat ? k_fused_pq<2, true> : k_fused_pq<2, false>), dim3(nb),
+               dim3(kThreads), smem, s, pdl, g, (const double*)c->tabS, (const double*)c->z, c->pb[0], c->pb[1], c->q,
+               x_lag_target(c), c->st, c->red, c->cnt + CNT_PQ);
 }
 
 // x[0..n) = v (start vectors of the convenience entry points)
@@ -1795,10 +1888,10 @@ __global__ void __launch_bounds__(kThreads, 6) kb_fused_pq(const BInst* __restri
   if (!I.active) return;
   double* x = lag ? I.x : nullptr;
   if (PAIRS)
-    fused_pq_pairs_body(VBlk{m.y, I.nb_fused}, I.g, I.tabS2, I.z, I.pb0, I.pb1, I.q, x, I.st, I.red,
+    fused_pq_pairs_body<false>(VBlk{m.y, I.nb_fused}, I.g, I.tabS2, I.z, I.pb0, I.pb1, I.q, x, I.st, I.red,
                         I.cnt + CNT_PQ);
   else
-    fused_pq_body<2>(VBlk{m.y, I.nb_fused}, I.g, I.tabS, I.z, I.pb0, I.pb1, I.q, x, I.st, I.red,
+    fused_pq_body<2, false>(VBlk{m.y, I.nb_fused}, I.g, I.tabS, I.z, I.pb0, I.pb1, I.q, x, I.st, I.red,
                      I.cnt + CNT_PQ);
 }
 
