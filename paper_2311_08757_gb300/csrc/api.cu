@@ -39,10 +39,10 @@ int guarded(dd_ctx* c, F&& f) {
     const int rc = f();
     // a bounded device wait that expired (tensor-core GEMM pipeline, coarse-solve copy) left
     // its bit in the error word; the results of that call cannot be trusted
-    if (rc == DD_OK && c != nullptr && c->dev_err != nullptr) {
-      int e = 0;
-      DD_CUDA(cudaMemcpyAsync(&e, c->dev_err + 8, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    if (rc == DD_OK && c != nullptr && c->err_h != nullptr) {
+      DD_CUDA(cudaMemcpyAsync(c->err_h, c->dev_err + 8, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
       DD_CUDA(cudaStreamSynchronize(c->stream));
+      const int e = *c->err_h;
       if (e != 0) {
         DD_CUDA(cudaMemsetAsync(c->dev_err + 8, 0, sizeof(int), c->stream));
         return fail(c, DD_ETIMEOUT, "a bounded device wait expired (code " + std::to_string(e) + ")");
@@ -492,9 +492,7 @@ int gmres_run(dd_ctx* c, const double* b, double rtol, int maxit, int* iters, do
     if (c->timing) timer_collect(c);
     return c->gm_res_h[0];
   };
-  PcgState init;
-  std::memset(&init, 0, sizeof(init));
-  DD_CUDA(cudaMemcpyAsync(c->st, &init, sizeof(init), cudaMemcpyHostToDevice, s));
+  DD_CUDA(cudaMemsetAsync(c->st, 0, sizeof(PcgState), s));
   // r_0 = b - A x_0
   TIMED(KC_STENCIL, s, launch_stencil(c, c->tabS, c->x, W, s));
   TIMED(KC_XRUPDATE, s, launch_axpby(c, -1.0, W, 1.0, nullptr, b, W, s));
@@ -706,9 +704,10 @@ int dd_setup(const dd_grid* gr, const double* V, size_t nV, void* stream, dd_ctx
     DD_CUDA(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
     DD_CUDA(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
     DD_CUDA(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
-    DD_CUDA(cudaMallocHost(&c->st_h, sizeof(PcgState)));
+    DD_CUDA(cudaMallocHost(&c->st_h, sizeof(PcgState) + sizeof(int)));
     DD_CUDA(cudaMallocHost(&c->ost_h, sizeof(OuterState)));
     c->dev_err = (int*)dev_alloc(c, sizeof(int) * 16);
+    c->err_h = reinterpret_cast<int*>(c->st_h + 1);
     c->red = (double*)dev_alloc(c, sizeof(double) * kMaxRedBlocks * 4);
     c->cnt = (unsigned*)dev_alloc(c, sizeof(unsigned) * CNT_NUM);
     c->st = (PcgState*)dev_alloc(c, sizeof(PcgState));
@@ -881,8 +880,7 @@ int dd_apply_operator(dd_ctx* c, int op, const double* x, double* y) {
     load_vec(c, x, c->w1);
     launch_stencil(c, tab, c->w1, c->w2, c->stream);
     store_vec(c, c->w2, y);
-    DD_CUDA(cudaStreamSynchronize(c->stream));
-    return DD_OK;
+    return DD_OK;   // guarded() waits for the stream
   });
 }
 
@@ -927,15 +925,15 @@ int dd_apply_preconditioner(dd_ctx* c, const double* r, double* z) {
   if (rc) return rc;
   return guarded(c, [&]() -> int {
     enter(c);
-    PcgState init;
-    std::memset(&init, 0, sizeof(init));
-    DD_CUDA(cudaMemcpyAsync(c->st, &init, sizeof(init), cudaMemcpyHostToDevice, c->stream));
+    DD_CUDA(cudaMemsetAsync(c->st, 0, sizeof(PcgState), c->stream));
     load_vec(c, r, c->r);
     precond(c, c->r, 0);
     store_vec(c, c->z, z);
-    DD_CUDA(cudaStreamSynchronize(c->stream));
-    if (c->timing) timer_collect(c);
-    return DD_OK;
+    if (c->timing) {
+      DD_CUDA(cudaStreamSynchronize(c->stream));
+      timer_collect(c);
+    }
+    return DD_OK;   // guarded() waits for the stream
   });
 }
 
@@ -1134,9 +1132,7 @@ int dd_lopcg(dd_ctx* c, double* x, int inner, double tol_res, double tol_lam, in
       const double* W = nullptr;
       int it = 0;
       if (inner == DD_INNER_FUSED) {
-        PcgState init;
-        std::memset(&init, 0, sizeof(init));
-        DD_CUDA(cudaMemcpyAsync(c->st, &init, sizeof(init), cudaMemcpyHostToDevice, s));
+        DD_CUDA(cudaMemsetAsync(c->st, 0, sizeof(PcgState), s));
         precond(c, RO, 0);
         W = c->z;
         it = 1;

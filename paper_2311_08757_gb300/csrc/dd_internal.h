@@ -285,6 +285,7 @@ struct dd_ctx {
   dd::PcgState* st = nullptr;
   dd::OuterState* ost = nullptr;
   dd::PcgState* st_h = nullptr;    // pinned mirror
+  int* err_h = nullptr;            // pinned, behind st_h: the error word after a call
   dd::OuterState* ost_h = nullptr; // pinned mirror
   dd::LopState* lst = nullptr;     // SI-LOPCG step scalars (device)
   dd::LopState* lst_h = nullptr;   // pinned mirror
