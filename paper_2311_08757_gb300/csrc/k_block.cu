@@ -706,9 +706,12 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
   }
 }
 
-// The launch shape.  Planes of at most 32 unknowns: PW warps per subdomain and side, by the pipe
-// time of the busiest sub-partition (2 nsub PW warps over 4 per SM, each cpp + PW - 1 + 4 FP64
-// instructions a plane): 4 up to about 75 subdomains, 2 up to about 150, then 1.  With PW = 1 the
+// The launch shape.  Planes of at most 32 unknowns: PW warps per subdomain and side, 4 while every
+// sub-partition gets one of them at most (2 nsub PW warps over 4 per SM: 76 subdomains), 2 while it gets
+// two (304), then 1.  A warp alone leaves most of its pipe idle, so two half-length products beside each other beat
+// one of full length, but a third starts another round (us per launch for 1 / 2 / 4: h = 1/32, L = 64
+// 72 / 48 / 42, L = 100 71 / 50 / 55, L = 301 84 / 66 / 123, L = 350 87 / 121 / 124; h = 1/20, l = 1.5,
+// L = 301 48 / 43 / 79, L = 350 49 / 76 / 78; h = 1/12, L = 200 24 / 22 / 30).  With PW = 1 the
 // blocks take 1, 2 or 4 subdomains: small blocks spread evenly over few rounds (us per launch for
 // 1 / 2 / 4 at h = 1/32: L = 512 88 / 96 / 96, L = 1000 187 / 158 / 177, L = 2048 361 / 353 / 319,
 // where four warps also share each plane's copy).
@@ -725,16 +728,7 @@ void block_groups(dd_ctx* c, int want) {
   const int RG = B.ms / 32, N = c->g.nsub, sms = 152;
   int cr = 1, PW = 1, RW = 1, rgl = 1, R = 1;
   if (RG == 1) {
-    int mmax = 1;
-    for (int t = 0; t < c->ntypes; ++t) mmax = std::max(mmax, B.w2[t] * c->g.nyi);
-    long long best = 0;
-    for (int q = 1; q <= 4; q *= 2) {
-      const long long cost = ((2LL * N * q + 4 * sms - 1) / (4 * sms)) * ((mmax + q - 1) / q + q + 3);
-      if (q == 1 || cost < best) {
-        best = cost;
-        PW = q;
-      }
-    }
+    PW = 8 * N <= 4 * sms ? 4 : (4 * N <= 8 * sms ? 2 : 1);
     const double x = 2.0 * N / (4 * sms);   // half chains per sub-partition
     R = std::min(want > 0 ? want : (x <= 2.0 ? 1 : (x <= 5.0 ? 2 : 4)), 4 / PW);
   } else {
