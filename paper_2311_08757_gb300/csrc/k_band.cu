@@ -149,8 +149,8 @@ __global__ void __launch_bounds__(1024) k_band_factor_win(T* CB, T* inv, const i
 // registers (rows over the lanes, Q per lane, the multipliers by shuffle), and the block applies
 // all eight to the trailing window with one read and write of each entry.  The columns that enter
 // are loaded a panel ahead.
-// Order 1209, band 32 (the three local types at L = 2048, n = 32): 549 -> 298 us; order 992, band 63
-// (its cell): 549 -> 330 us.
+// Order 1209, band 32 (the three local types at L = 2048, n = 32): 549 -> 272 us; order 992, band 63
+// (its cell): 549 -> 316 us.
 constexpr int kPb = 8;
 template <int Q, int PPT>
 __global__ void __launch_bounds__(Q <= 3 ? 512 : 1024) k_band_factor_panel(float* CB, float* inv, const int* __restrict__ nvec,
