@@ -502,19 +502,15 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
                                                          int kpad, const PcgState* st, int* err) {
   constexpr int CPP = 32 / PW, MS = 32, NT = (P == 1) ? 3 : 9, D = row_stages(PW);
   if (st != nullptr && st->done) return;
-  cluster_arrive();
   extern __shared__ __align__(128) double s_ring[];  // [D][32][32]
   __shared__ __align__(16) double s_g[4][32];        // per warp: the product's argument
   __shared__ double s_part[2][4][32];                // partial sums, alternating
   __shared__ double s_mid[4][32];                    // left side: B h_{t+1}; right side: x_t
   __shared__ __align__(8) unsigned long long s_bar[2 * D + 4];   // full, empty, meeting
-  const int side = (int)cluster_rank();
-  const int2 grp = groups[blockIdx.x >> 1];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5) - 1;   // nw working warps
-  const int ty = subs[sub_of_slot[grp.x]].type, K = B.w1[ty], t = K / 2;
-  const int nmine = side ? K - 1 - t : t, k0 = side ? K - 1 : 0, dir = side ? -1 : 1;
-  const int nprod = 2 * nmine + (side ? 0 : 1);      // products: inwards, plane t (left side), outwards
   const uint32_t bar = smem_u32(s_bar);
+  // The barriers exist before any thread arrives, so the cluster barrier's release and acquire show
+  // them to both blocks: the other side's first arrival at the meeting may follow its wait at once.
   if (threadIdx.x == 0) {
     for (int i = 0; i < D; ++i) {
       mbar_init(bar + 8 * i, 1);
@@ -524,7 +520,12 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  __syncthreads();
+  cluster_arrive();
+  const int side = (int)cluster_rank();
+  const int2 grp = groups[blockIdx.x >> 1];
+  const int ty = subs[sub_of_slot[grp.x]].type, K = B.w1[ty], t = K / 2;
+  const int nmine = side ? K - 1 - t : t, k0 = side ? K - 1 : 0, dir = side ? -1 : 1;
+  const int nprod = 2 * nmine + (side ? 0 : 1);      // products: inwards, plane t (left side), outwards
   cluster_wait();
   if (w == nw) {   // the ring's producer
     if (lane == 0)
