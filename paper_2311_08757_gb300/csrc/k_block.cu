@@ -528,8 +528,9 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
   const int nprod = 2 * nmine + (side ? 0 : 1);      // products: inwards, plane t (left side), outwards
   cluster_wait();
   if (w == nw) {   // the ring's producer
-    if (lane == 0)
-      for (int q = 0; q < nprod; ++q) {
+    if (lane == 0) {
+      int q = 0;
+      for (; q < nprod; ++q) {
         const int sl = q % D;
         if (q >= D && !mbar_wait(bar + 8 * (D + sl), (uint32_t)(q / D - 1) & 1u, err, ERR_BLK_WAIT)) break;
         const int i = q < nmine ? q : 2 * nmine - q - (side ? 1 : 0);   // plane i from this side's end (nmine: t)
@@ -537,6 +538,10 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
         bulk_g2s(smem_u32(s_ring + sl * MS * MS), blk_inverse(B, Sinv, ty, k0 + dir * i), MS * MS * sizeof(double),
                  bar + 8 * sl);
       }
+      // the last copy into each slot: a warp that gave up has not waited for it
+      for (int k = max(0, q - D); k < q; ++k) mbar_wait(bar + 8 * (k % D), (uint32_t)(k / D) & 1u, err, ERR_BLK_WAIT);
+    }
+    cluster_sync_all();
     return;
   }
   const int rr = w / PW, pw = w % PW;
@@ -705,6 +710,9 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
       load_cf(pl(max(i - 1, 0)), dir, c1);
     }
   }
+  // On every path, also after a wait that gave up (its warp runs through the remaining, meaningless work
+  // without waiting): the other block's stores into this one have landed before it ends.
+  cluster_sync_all();
 }
 
 // The launch shape.  Planes of at most 32 unknowns: PW warps per subdomain and side, 4 while every
