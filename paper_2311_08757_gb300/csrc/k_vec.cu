@@ -1156,14 +1156,13 @@ __global__ void __launch_bounds__(kClsThreads, 3) k_matvec_pq_pairs_cls(Geo g, c
   const double* __restrict__ p = p_cur(pb0, pb1, st->iter);
   double acc[1] = {0.0};
   int sl = 0, ph = 0;
-  bool dead = false;   // a wait gave up: the error word tells the host
   __syncthreads();
   for (int it = kb; it < nitem; it += nbr) {
     // the stage read two steps ago is free: every thread has passed the barrier that ended that step
     if (threadIdx.x == 0 && it + (kClsStages - 1) * nbr < nitem)
       fetch(it + (kClsStages - 1) * nbr, sl == 0 ? kClsStages - 1 : sl - 1);
-    if (!dead && !mbar_wait(bar + 8 * sl, (uint32_t)ph, err, ERR_MATVEC_WAIT)) dead = true;
-    if (mine) {
+    const bool here = mbar_wait(bar + 8 * sl, (uint32_t)ph, err, ERR_MATVEC_WAIT);
+    if (mine && here) {
       const int a1 = a1_first + n * (it / nset), col = kClsPairs * n * (it % nset) + c0 + cl;   // in the first pair
       const long long idx = (long long)a1 * c1 + ((long long)col << yl) + slot;
       bool ok[2 * kClsPairs];
@@ -1205,7 +1204,16 @@ __global__ void __launch_bounds__(kClsThreads, 3) k_matvec_pq_pairs_cls(Geo g, c
       sl = 0;
       ph ^= 1;
     }
-    __syncthreads();
+    if (__syncthreads_or(!here)) {
+      // a wait gave up (the error word tells the host): no further step, and no copy outlives the block
+      if (threadIdx.x == 0)
+        for (int i = it; i < min(nitem, it + kClsStages * nbr); i += nbr) {   // the items fetched so far
+          const int k = (i - kb) / nbr;
+          mbar_wait(bar + 8 * (k % kClsStages), (uint32_t)(k / kClsStages) & 1u, err, ERR_MATVEC_WAIT);
+        }
+      __syncthreads();
+      break;
+    }
   }
   double tot[1];
   if (grid_sum_last<1>(acc, partials, counter, tot) && threadIdx.x == 0) {
