@@ -358,7 +358,7 @@ void launch_check_finite(const double* v, long long n, int* flag, cudaStream_t s
 // ----------------------------------------------------------------------------------------
 
 // stencil_at where x is mostly zero: a warp whose taps all read zeros has the value 0 without its
-// products.  A solve usually starts from x = 0, and the FP64 pipe bounds the stencil (p = 2: 27
+// products.  All lanes of the warp call it together.  A solve usually starts from x = 0, and the FP64 pipe bounds the stencil (p = 2: 27
 // products per node; L = 64, h = 1/16 from zero: 830 -> 248 us).
 template <int P>
 __device__ __forceinline__ double stencil_unless_zero(const Geo& g, const double* __restrict__ tab,
@@ -371,7 +371,7 @@ __device__ __forceinline__ double stencil_unless_zero(const Geo& g, const double
     const double v = x[idx + d1 * c1 + d2 * c2 + dy];
     any |= ((unsigned)__double2hiint(v) << 1) | (unsigned)__double2loint(v);
   }
-  return __any_sync(__activemask(), any != 0u) ? stencil_at<P>(g, tab, x, idx, cls) : 0.0;
+  return __any_sync(kFull, any != 0u) ? stencil_at<P>(g, tab, x, idx, cls) : 0.0;
 }
 
 // r = b - A_sigma x, rr0 = (r, r), tol2 = rtol^2 rr0 (rtol^2 preset in tol2 by the host).
@@ -382,13 +382,16 @@ __device__ __forceinline__ void pcg_init_body(VBlk vb, Geo g, const double* __re
                                                        PcgState* st, double* partials, unsigned* counter) {
   const long long total = (long long)g.nxi * (P == 2 ? g.nxi : 1) * g.Ypad;
   double acc[1] = {0.0};
-  for (long long t = (long long)vb.b * blockDim.x + threadIdx.x; t < total;
+  const int lane = threadIdx.x & 31;
+  for (long long t = (long long)vb.b * blockDim.x + threadIdx.x; t - lane < total;   // whole warps
        t += (long long)vb.nb * blockDim.x) {
-    Node nd = node_of<P>(g, t);
+    Node nd = node_of<P>(g, min(t, total - 1));
     const int cls = cls_of<P>(g, nd);
     const double v = b[nd.idx] - stencil_unless_zero<P>(g, tab, x, nd.idx, cls);
-    r[nd.idx] = v;
-    acc[0] = fma(v, v, acc[0]);
+    if (t < total) {
+      r[nd.idx] = v;
+      acc[0] = fma(v, v, acc[0]);
+    }
   }
   double tot[1];
   if (grid_sum_last<1>(acc, partials, counter, tot, vb) && threadIdx.x == 0) {
