@@ -343,6 +343,11 @@ int dd_apply_asigma_pairs(dd_ctx* ctx, const double* x, double* y);
  * needs dd_coarse_build. */
 int dd_apply_preconditioner(dd_ctx* ctx, const double* r, double* z);
 
+/* (r, r) as the stop test of the context's last PCG iteration saw it, and (r_0, r_0) (host
+ * doubles; zero after a call that left no PCG state); needs dd_coarse_build.  A batch and a single
+ * call leave the same bits. */
+int dd_pcg_residual(dd_ctx* ctx, double* rr, double* rr0);
+
 /* Coarse matrix A_{sigma,0} = R_0 A_sigma R_0^T copied to host as a dense nsub x nsub
  * row-major array (needs dd_coarse_build; grid.coarse = 1). */
 int dd_coarse_matrix(dd_ctx* ctx, double* A0_host);

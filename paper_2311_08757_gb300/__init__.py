@@ -83,6 +83,7 @@ _SIGS = {
     "dd_apply_operator": (c_int, [c_void_p, c_int, c_void_p, c_void_p]),
     "dd_apply_asigma_pairs": (c_int, [c_void_p, c_void_p, c_void_p]),
     "dd_apply_preconditioner": (c_int, [c_void_p, c_void_p, c_void_p]),
+    "dd_pcg_residual": (c_int, [c_void_p, POINTER(c_double), POINTER(c_double)]),
     "dd_coarse_matrix": (c_int, [c_void_p, c_void_p]),
     "dd_set_option": (c_int, [c_void_p, c_int, c_int]),
     "dd_kernel_timings": (c_int, [c_void_p, POINTER(c_int), POINTER(c_char_p), POINTER(c_longlong),
@@ -263,6 +264,13 @@ def dd_apply_operator(ctx, op: int, x, y) -> None:
 def dd_apply_asigma_pairs(ctx, x, y) -> None:
     """y = A_sigma x by the float-pair pass of the PCG iteration (see the header)."""
     _check(lib().dd_apply_asigma_pairs(ctx, _ptr(x), _ptr(y)), ctx)
+
+
+def dd_pcg_residual(ctx):
+    """(r, r) and (r_0, r_0) of the context's last PCG solve."""
+    rr, rr0 = c_double(), c_double()
+    _check(lib().dd_pcg_residual(ctx, byref(rr), byref(rr0)), ctx)
+    return rr.value, rr0.value
 
 
 def dd_apply_preconditioner(ctx, r, z) -> None:

@@ -362,9 +362,14 @@ bool fuse_xr_possible(const dd_ctx* c) {
 // n = 32: L = 37 39.5 -> 37.9 us, L = 256 43.0 -> 40.6, L = 512 49.5 -> 48.0, but L = 1024 64.9 -> 65.5 and
 // L = 2048 95.7 -> 100.8 us; n = 12: L = 37 30.8 -> 28.5, L = 512 35.1 -> 33.8, L = 1024 39.6 -> 40.2 us.
 constexpr int kFuseXrMaxSub = 512;
+
+}  // namespace
+
 bool fuse_xr(const dd_ctx* c) {
   return c->fuse_xr || (c->fuse_xr_opt < 0 && fuse_xr_possible(c) && c->g.nsub <= kFuseXrMaxSub);
 }
+
+namespace {
 
 void pcg_iteration(dd_ctx* c) {
   cudaStream_t s = c->stream;
@@ -934,6 +939,20 @@ int dd_apply_preconditioner(dd_ctx* c, const double* r, double* z) {
       timer_collect(c);
     }
     return DD_OK;   // guarded() waits for the stream
+  });
+}
+
+int dd_pcg_residual(dd_ctx* c, double* rr, double* rr0) {
+  if (!rr || !rr0) return fail(c, DD_EINVAL, "null pointer");
+  int rc = stage_err(c, 3);
+  if (rc) return rc;
+  return guarded(c, [&]() -> int {
+    enter(c);
+    DD_CUDA(cudaMemcpyAsync(c->st_h, c->st, sizeof(PcgState), cudaMemcpyDeviceToHost, c->stream));
+    DD_CUDA(cudaStreamSynchronize(c->stream));
+    *rr = c->st_h->rr;
+    *rr0 = c->st_h->rr0;
+    return DD_OK;
   });
 }
 

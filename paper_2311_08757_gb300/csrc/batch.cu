@@ -45,14 +45,14 @@ struct BGroup {
   std::vector<BInst> Bh;
   BInst* B = nullptr;
   int2 *vm_init = nullptr, *vm_fused = nullptr, *vm_xr = nullptr, *vm_prolong = nullptr, *vm_sdot = nullptr,
-       *vm_st = nullptr, *vm_st2 = nullptr, *vm_vec = nullptr, *vm_pack = nullptr, *vm_lop = nullptr;
-  int n_init = 0, n_fused = 0, n_xr = 0, n_prolong = 0, n_sdot = 0, n_st = 0, n_st2 = 0, n_vec = 0, n_pack = 0, n_lop = 0;
+       *vm_st = nullptr, *vm_st2 = nullptr, *vm_vec = nullptr, *vm_pack = nullptr, *vm_lop = nullptr, *vm_xs = nullptr;
+  int n_init = 0, n_fused = 0, n_xr = 0, n_prolong = 0, n_sdot = 0, n_st = 0, n_st2 = 0, n_vec = 0, n_pack = 0, n_lop = 0, n_xs = 0;
   size_t cr_smem = 0;
   int ypad = 0, precision = 0, check_every = 8;
   bool arith = true;               // every instance's prolong-sum owners in closed form
   bool pairs = false;              // q = A_sigma p in float pairs (the same choice for every instance)
   bool lag = false;                // x updated one iteration late, by the p update (the same for every instance)
-  bool fuse = false;               // the x/r update inside the packing (the same for every instance)
+  bool fuse = false;               // the x/r update inside the packing (option 1, the same for every instance)
   dd::BGemm* gemm = nullptr;
   int bn = 0;                      // N tile of the grouped contraction (timed at build)
   cudaStream_t s = nullptr, side = nullptr;
@@ -101,6 +101,7 @@ void free_group(BGroup* g) {
   dd::bgemm_destroy(g->gemm);
   for (void* p : {(void*)g->B, (void*)g->vm_init, (void*)g->vm_fused, (void*)g->vm_xr, (void*)g->vm_prolong,
                   (void*)g->vm_sdot, (void*)g->vm_st, (void*)g->vm_st2, (void*)g->vm_vec, (void*)g->vm_pack, (void*)g->vm_lop,
+                  (void*)g->vm_xs,
                   (void*)g->stat_d, (void*)g->xptr_d, (void*)g->err_d})
     if (p) cudaFree(p);
   if (g->stat_h) cudaFreeHost(g->stat_h);
@@ -116,7 +117,7 @@ void free_group(BGroup* g) {
 long long option_signature(const dd_batch* b) {
   long long h = 1469598103934665603LL;
   for (const dd_ctx* c : b->ctx)
-    for (int v : {c->prolong_arith, c->pq_pairs, c->fuse_xr, c->x_lag, c->flexible_opt, c->check_every, c->gemm_bn_opt})
+    for (int v : {c->prolong_arith, c->pq_pairs, c->fuse_xr, (int)fuse_xr(c), c->x_lag, c->flexible_opt, c->check_every, c->gemm_bn_opt})
       h = (h ^ (long long)(v + 7)) * 1099511628211LL;
   return h;
 }
@@ -192,7 +193,8 @@ void pcg_iteration(BGroup* g) {
     dd::launch_b_pack_xr(g->B, g->vm_pack, g->n_pack, g->precision, g->s);
     precond(g, 2, true);
   } else {
-    dd::launch_b_xr_update(g->B, g->vm_xr, g->n_xr, g->lag, g->s);
+    if (g->n_xr > 0) dd::launch_b_xr_update(g->B, g->vm_xr, g->n_xr, g->lag, g->s);
+    if (g->n_xs > 0) dd::launch_b_xr_update_sub(g->B, g->vm_xs, g->n_xs, g->lag, g->s);
     precond(g, 2);
   }
 }
@@ -245,7 +247,7 @@ BGroup* build_group(dd_batch* b, const std::vector<int>& idx) {
     DD_CUDA(cudaMalloc(&g->err_d, sizeof(int) * 16));
     DD_CUDA(cudaMemset(g->err_d, 0, sizeof(int) * 16));
     g->Bh.assign(n, BInst());
-    std::vector<int2> vinit, vfused, vxr, vprol, vsdot, vst, vst2, vvec, vpack, vlop;
+    std::vector<int2> vinit, vfused, vxr, vprol, vsdot, vst, vst2, vvec, vpack, vlop, vxs;
     std::vector<dd_ctx*> cs;
     std::vector<int> tb, sb;
     std::vector<double*> xs;
@@ -284,10 +286,11 @@ BGroup* build_group(dd_batch* b, const std::vector<int>& idx) {
       I.ptypes = c->ptypes;
       I.prolong_arith = c->prolong_arith;
       g->arith = g->arith && c->prolong_arith;
+      I.sub_rr = fuse_xr(c) ? 1 : 0;
       dd::batch_grid_sizes(c, &I);
       for (int k = 0; k < I.nb_init; ++k) vinit.push_back(make_int2(j, k));
       for (int k = 0; k < I.nb_fused; ++k) vfused.push_back(make_int2(j, k));
-      for (int k = 0; k < I.nb_xr; ++k) vxr.push_back(make_int2(j, k));
+      for (int k = 0; k < (I.sub_rr ? I.nsub : I.nb_xr); ++k) (I.sub_rr ? vxs : vxr).push_back(make_int2(j, k));
       for (int k = 0; k < I.nb_prolong; ++k) vprol.push_back(make_int2(j, k));
       for (int k = 0; k < I.nb_sdot; ++k) vsdot.push_back(make_int2(j, k));
       for (int k = 0; k < I.nb_st; ++k) vst.push_back(make_int2(j, k));
@@ -301,6 +304,7 @@ BGroup* build_group(dd_batch* b, const std::vector<int>& idx) {
     g->vm_init = upload_vmap(vinit); g->n_init = (int)vinit.size();
     g->vm_fused = upload_vmap(vfused); g->n_fused = (int)vfused.size();
     g->vm_xr = upload_vmap(vxr); g->n_xr = (int)vxr.size();
+    g->vm_xs = upload_vmap(vxs); g->n_xs = (int)vxs.size();
     g->vm_prolong = upload_vmap(vprol); g->n_prolong = (int)vprol.size();
     g->vm_sdot = upload_vmap(vsdot); g->n_sdot = (int)vsdot.size();
     g->vm_st = upload_vmap(vst); g->n_st = (int)vst.size();

@@ -120,6 +120,31 @@ __device__ __forceinline__ const double* p_prev(const double* pb0, const double*
 }
 __device__ __forceinline__ double* p_cur(double* pb0, double* pb1, int k) { return (k & 1) ? pb0 : pb1; }
 
+// end of a PCG iteration's x/r update: rr = (r, r), and the stop test on it
+__device__ __forceinline__ void pcg_stop_test(PcgState* st, double rr) {
+  st->rr = rr;
+  st->iter += 1;
+  if (!isfinite(rr)) {
+    st->status = DD_ENAN;
+    st->done = 1;
+  } else if (rr <= st->tol2) {
+    st->done = 1;
+  } else if (st->iter >= st->maxit) {
+    st->status = DD_EMAXIT;
+    st->done = 1;
+  }
+}
+
+// p = 1: the node columns a with min(a / n, L - 1) = s, so that each column belongs to one subdomain, as
+// pairs of entries lo <= e < hi counted from the subdomain's first column lo1
+struct OwnedRun {
+  int lo, hi;
+};
+__device__ __forceinline__ OwnedRun owned_run(const Geo& g, int s, int lo1) {
+  const int a_lo = max(1, s * g.n), a_hi = (s == g.L - 1) ? g.nxi : (s + 1) * g.n - 1;
+  return OwnedRun{(a_lo - lo1) * g.Ypad / 2, (a_hi + 1 - lo1) * g.Ypad / 2};
+}
+
 // A block's place in the launch of one problem: block b of nb.  A plain launch is one
 // problem (b = blockIdx.x, nb = gridDim.x); a batched launch runs the blocks of several
 // problems' launches side by side, each block with the index and count it would have had

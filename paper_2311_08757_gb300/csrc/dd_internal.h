@@ -301,6 +301,9 @@ struct dd_ctx {
 // the x that the PCG p update advances (x_lag), or null when the x/r update does it
 inline double* x_lag_target(dd_ctx* c) { return c->x_lag ? c->x : nullptr; }
 
+// whether the PCG iteration of this context's own solves fuses the x/r update into the packing
+bool fuse_xr(const dd_ctx* c);
+
 namespace dd {
 
 // One problem of a batched launch: its geometry, the device buffers of its context, and the
@@ -341,6 +344,7 @@ struct BInst {
   double* lop_red;
   int4 ptypes;            // p = 1: type ids of the left end, interior and right end subdomains
   int prolong_arith;      // the prolong-sum's owners computed in closed form (p = 1)
+  int sub_rr;             // (r, r) added up by subdomains: the plain solve fuses the x/r update into the packing
 };
 
 // Vector roles in BInst (the batched outer-step kernels take roles, not pointers);
@@ -356,6 +360,7 @@ struct BStat {
 };
 
 // ----- launchers (kernels in k_*.cu) -----
+constexpr int kPackThreads = 128;   // restriction packing, one block per subdomain
 int grid_blocks(long long work, int threads, int max_per_sm = 8);
 int lop_blocks(long long n);   // SI-LOPCG update pass over n entries
 
@@ -452,6 +457,7 @@ void launch_b_zero_pcg(const BInst* B, const int2* vmap, int nvb, cudaStream_t s
 void launch_b_pcg_init(const BInst* B, const int2* vmap, int nvb, int b_role, cudaStream_t s);
 void launch_b_fused_pq(const BInst* B, const int2* vmap, int nvb, int ypad, bool pairs, bool lag, cudaStream_t s);
 void launch_b_xr_update(const BInst* B, const int2* vmap, int nvb, bool lag, cudaStream_t s);
+void launch_b_xr_update_sub(const BInst* B, const int2* vmap, int nvb, bool lag, cudaStream_t s);   // sub_rr instances
 void launch_b_x_final(const BInst* B, const int2* vmap, int nvb, cudaStream_t s);   // after lagged x updates
 void launch_b_prolong(const BInst* B, const int2* vmap, int nvb, int mode, bool arith, bool upd, cudaStream_t s);
 void launch_b_pack_xr(const BInst* B, const int2* vmap, int nvb, int precision, cudaStream_t s);

@@ -491,8 +491,7 @@ __device__ __forceinline__ void pack_xr_body(VBlk vb, Geo g, const Sub* __restri
   const int Y = g.Ypad;
   const int npair = sb.w1 * Y / 2;   // p = 1: the restriction is one run of w1 columns
   const long long g0 = (long long)sb.lo1 * Y;
-  const int own_lo = max(1, s * g.n), own_hi = (s == g.L - 1) ? g.nxi : (s + 1) * g.n - 1;
-  const int e_lo = (own_lo - sb.lo1) * Y / 2, e_hi = (own_hi + 1 - sb.lo1) * Y / 2;
+  const OwnedRun own = owned_run(g, s, sb.lo1);
   double rr[1] = {0.0}, acc[1] = {0.0};
   for (int e = threadIdx.x; e < npair; e += blockDim.x) {
     const int kp = 2 * e;
@@ -501,7 +500,7 @@ __device__ __forceinline__ void pack_xr_body(VBlk vb, Geo g, const Sub* __restri
     const double2 qv = *reinterpret_cast<const double2*>(q + gi);
     rv.x = fma(-alpha, qv.x, rv.x);
     rv.y = fma(-alpha, qv.y, rv.y);
-    if (e >= e_lo && e < e_hi) {
+    if (e >= own.lo && e < own.hi) {
       if (x != nullptr) {   // null: the next p update makes it (x_lag)
         const double2 pv = *reinterpret_cast<const double2*>(p + gi);
         double2 xv = *reinterpret_cast<const double2*>(x + gi);
@@ -523,20 +522,7 @@ __device__ __forceinline__ void pack_xr_body(VBlk vb, Geo g, const Sub* __restri
     if (threadIdx.x == 0) c0[s] = acc[0];
   }
   double tot[1];
-  if (grid_sum_last<1>(rr, partials, counter, tot, vb) && threadIdx.x == 0) {
-    const double rrv = tot[0];
-    st->rr = rrv;
-    st->iter += 1;
-    if (!isfinite(rrv)) {
-      st->status = DD_ENAN;
-      st->done = 1;
-    } else if (rrv <= st->tol2) {
-      st->done = 1;
-    } else if (st->iter >= st->maxit) {
-      st->status = DD_EMAXIT;
-      st->done = 1;
-    }
-  }
+  if (grid_sum_last<1>(rr, partials, counter, tot, vb) && threadIdx.x == 0) pcg_stop_test(st, tot[0]);
 }
 
 template <typename T>
@@ -840,7 +826,6 @@ int gemm_setup(dd_ctx* c) {
 // 128 threads (16 blocks of 31 registers per SM): all 2048 subdomain blocks of the
 // L = 2048, h = 1/32 box are resident at once instead of 1216 + 832 blocks of 256 (14.3
 // against 15.6 us)
-constexpr int kPackThreads = 128;
 
 void launch_pack(dd_ctx* c, const double* r, double* c0, cudaStream_t s) {
   const Geo& g = c->g;

@@ -1297,20 +1297,46 @@ __device__ __forceinline__ void xr_update_body(VBlk vb, long long n, double* pb0
     acc[0] = fma(rv.y, rv.y, acc[0]);
   }
   double tot[1];
-  if (grid_sum_last<1>(acc, partials, counter, tot, vb) && threadIdx.x == 0) {
-    const double rr = tot[0];
-    st->rr = rr;
-    st->iter += 1;
-    if (!isfinite(rr)) {
-      st->status = DD_ENAN;
-      st->done = 1;
-    } else if (rr <= st->tol2) {
-      st->done = 1;
-    } else if (st->iter >= st->maxit) {
-      st->status = DD_EMAXIT;
-      st->done = 1;
+  if (grid_sum_last<1>(acc, partials, counter, tot, vb) && threadIdx.x == 0) pcg_stop_test(st, tot[0]);
+}
+
+// The same update by blocks of 128 threads, one per subdomain: (r, r) is added up exactly as the packing
+// with the fused update adds it (pack_xr_body), so that a batch takes the steps that the single
+// solve of a box with the fused form takes.
+template <bool UPX>
+__device__ __forceinline__ void xr_update_sub_body(VBlk vb, Geo g, const Sub* __restrict__ subs, double* pb0,
+                                                   double* pb1, const double* __restrict__ q, double* __restrict__ x,
+                                                   double* __restrict__ r, PcgState* st, double* partials,
+                                                   unsigned* counter) {
+  if (st->done) return;
+  const double alpha = st->alpha;
+  const int lo1 = subs[vb.b].lo1;
+  const OwnedRun own = owned_run(g, vb.b, lo1);
+  const long long first = (long long)lo1 * g.Ypad / 2;
+  const double2* p2 = reinterpret_cast<const double2*>(p_cur(pb0, pb1, st->iter)) + first;
+  const double2* q2 = reinterpret_cast<const double2*>(q) + first;
+  double2* x2 = reinterpret_cast<double2*>(x) + first;
+  double2* r2 = reinterpret_cast<double2*>(r) + first;
+  const int T = (int)blockDim.x, tid = (int)threadIdx.x;
+  double rr[1] = {0.0};
+  for (int e = tid + (max(own.lo - tid, 0) + T - 1) / T * T; e < own.hi; e += T) {
+    const double2 qv = q2[e];
+    double2 rv = r2[e];
+    if (UPX) {
+      const double2 pv = p2[e];
+      double2 xv = x2[e];
+      xv.x = fma(alpha, pv.x, xv.x);
+      xv.y = fma(alpha, pv.y, xv.y);
+      x2[e] = xv;
     }
+    rv.x = fma(-alpha, qv.x, rv.x);
+    rv.y = fma(-alpha, qv.y, rv.y);
+    r2[e] = rv;
+    rr[0] = fma(rv.x, rv.x, rr[0]);
+    rr[0] = fma(rv.y, rv.y, rr[0]);
   }
+  double tot[1];
+  if (grid_sum_last<1>(rr, partials, counter, tot, vb) && threadIdx.x == 0) pcg_stop_test(st, tot[0]);
 }
 
 template <bool UPX>
@@ -1914,6 +1940,16 @@ __global__ void __launch_bounds__(kThreads) kb_xr_update(const BInst* __restrict
   xr_update_body<UPX>(VBlk{m.y, I.nb_xr}, I.g.plen, I.pb0, I.pb1, I.q, I.x, I.r, I.st, I.red, I.cnt + CNT_RR);
 }
 
+// instances whose own solve fuses the x/r update into the packing (sub_rr)
+template <bool UPX>
+__global__ void __launch_bounds__(kPackThreads) kb_xr_update_sub(const BInst* __restrict__ B,
+                                                                 const int2* __restrict__ vmap) {
+  const int2 m = vmap[blockIdx.x];
+  const BInst& I = B[m.x];
+  if (!I.active) return;
+  xr_update_sub_body<UPX>(VBlk{m.y, I.nsub}, I.g, I.subs, I.pb0, I.pb1, I.q, I.x, I.r, I.st, I.red, I.cnt + CNT_RR);
+}
+
 // after the running instances' solves, with the lagged x update (two groups at once, 12 instances of
 // 25 to 512 cells, n = 32: the x/r update 17.3 -> 12.8 us, the p update 23.6 -> 24.0)
 __global__ void __launch_bounds__(kThreads) kb_x_final(const BInst* __restrict__ B, const int2* __restrict__ vmap) {
@@ -2138,6 +2174,12 @@ void launch_b_fused_pq(const BInst* B, const int2* vmap, int nvb, int ypad, bool
 void launch_b_xr_update(const BInst* B, const int2* vmap, int nvb, bool lag, cudaStream_t s) {
   if (lag) (kb_xr_update<false><<<nvb, kThreads, 0, s>>>(B, vmap), dd::note_launch());
   else (kb_xr_update<true><<<nvb, kThreads, 0, s>>>(B, vmap), dd::note_launch());
+  DD_CUDA(cudaGetLastError());
+}
+
+void launch_b_xr_update_sub(const BInst* B, const int2* vmap, int nvb, bool lag, cudaStream_t s) {
+  if (lag) (kb_xr_update_sub<false><<<nvb, kPackThreads, 0, s>>>(B, vmap), dd::note_launch());
+  else (kb_xr_update_sub<true><<<nvb, kPackThreads, 0, s>>>(B, vmap), dd::note_launch());
   DD_CUDA(cudaGetLastError());
 }
 
