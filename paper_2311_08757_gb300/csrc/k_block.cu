@@ -12,7 +12,8 @@
 //   h_k = S_k^{-1} (f_k - B h_{k -+ 1})  towards t,   x_t = h_t,   x_k = h_k - S_k^{-1} (B x_{k +- 1})
 // away from it: K steps of one dense m x m product each, where the banded triangular sweeps
 // took 2 K m dependent steps.  The work is 2 m^2 multiply-adds per plane and sweep pair
-// against 2 m (m + 1) for the banded factor, so nothing is paid for the shorter chain.
+// against 2 m (m + 1) for the banded factor.  On the pipe the rows come in warps of 32 and the columns in
+// chunks of 8 (4 for planes of at most 32 unknowns); the sweeps paid by the band's warps of 32.
 #include <algorithm>
 
 #include "dd_async.cuh"
@@ -20,10 +21,10 @@
 namespace dd {
 
 // Planes of the types' local boxes: type ty has K = w1 planes of m = w2 nyi unknowns; inverse
-// Schur complements are ms x ms, ms the largest m rounded up to whole warps (rows and columns
+// Schur complements are ms x ms, ms the largest m (mmax) rounded up to whole warps (rows and columns
 // past m hold the identity).
 struct BlkGeo {
-  int ntypes, ms, kmax;
+  int ntypes, ms, mmax, kmax;
   int w1[kMaxTypes], w2[kMaxTypes], lo1[kMaxTypes], lo2[kMaxTypes];
 };
 
@@ -203,17 +204,17 @@ __global__ void __launch_bounds__(kGjThreads) k_gj_panel(BlkGeo B, const double*
 static BlkGeo blk_geo(const dd_ctx* c) {
   BlkGeo B{};
   B.ntypes = c->ntypes;
-  int mmax = 1;
+  B.mmax = 1;
   for (int t = 0; t < c->ntypes; ++t) {
     B.w1[t] = c->type_w1[t];
     B.w2[t] = c->type_w2[t];
     B.kmax = std::max(B.kmax, B.w1[t]);
-    mmax = std::max(mmax, B.w2[t] * c->g.nyi);
+    B.mmax = std::max(B.mmax, B.w2[t] * c->g.nyi);
     const Sub& s = c->subs_h[c->rep_of_type[t]];
     B.lo1[t] = s.lo1;
     B.lo2[t] = s.lo2;
   }
-  B.ms = (mmax + 31) / 32 * 32;
+  B.ms = (B.mmax + 31) / 32 * 32;
   return B;
 }
 
@@ -260,6 +261,8 @@ void block_factor(dd_ctx* c, int* flag) {
 // ----------------------------------------------------------------------------------------
 struct BlkShape {
   int R, PW, RW, rgl;   // subdomains, column ranges and row warps per block; row groups per block
+  int nch, cpp;         // chunks of eight columns and columns of a range: the PW ranges cover mmax, not
+                        // ms, whose further columns meet zeros
 };
 
 __device__ __forceinline__ unsigned cluster_rank() {
@@ -331,7 +334,7 @@ __global__ void __launch_bounds__(1024) k_block_solve(Geo g, BlkGeo B, BlkShape 
   double* ub = sm + (size_t)(3 * R + rr) * ms;
   double* part = sm + (size_t)4 * R * ms + (size_t)rr * sh.PW * sh.rgl * 32;
   const int lane = tr & 31, w = tr >> 5, rw = w % sh.RW, pw = w / sh.RW;
-  const int cpp = ms / sh.PW, nch = cpp / 8;        // columns and 8-column chunks of this warp's range
+  const int cpp = sh.cpp, nch = sh.nch;             // columns and 8-column chunks of this warp's range
   const int rg_first = cr * sh.rgl + rw, rg_end = min((cr + 1) * sh.rgl, ms >> 5);
   const long long cstride = (P == 1) ? g.Ypad : (long long)g.ncx * g.Ypad;
   const double* rb = r + ((P == 1) ? (long long)sb.lo1 * g.Ypad : ((long long)sb.lo1 * g.ncx + sb.lo2) * g.Ypad);
@@ -724,14 +727,18 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
 // blocks take 1, 2 or 4 subdomains: small blocks spread evenly over few rounds (us per launch for
 // 1 / 2 / 4 at h = 1/32: L = 512 88 / 96 / 96, L = 1000 187 / 158 / 177, L = 2048 361 / 353 / 319,
 // where four warps also share each plane's copy).
-// Larger planes (k_block_solve): one subdomain per block, at most 20 warps, more blocks per side
-// while the grid does not fill the SMs.  The results do not depend on the subdomains per block.
+// Larger planes (k_block_solve): a warp per 32 rows, up to 4 subdomains and 32 warps per block, up to 4 column
+// ranges while that leaves an SM sub-partition at most 5 warps, up to 4 blocks per side while the grid
+// does not fill the SMs.  The results do not depend on the subdomains per block.
 //
 // Measured against the banded triangular sweeps this replaced (one warp per one or two
 // subdomains, 2 n_loc dependent steps; us per application): p = 1, h = 1/32, delta = 4: L = 32
 // 375 -> 36, L = 512 376 -> 88, L = 2048 434 -> 319 (the FP64 pipe needs 288 for its instructions);
 // ell = 2, L = 300 1327 -> 209; p = 2, h = 1/16, delta = 2 (planes of 285): L = 6 5667 -> 292,
 // L = 16 5689 -> 1604 (pipe floor of the banded flops 1330).
+// Planes of m unknowns stored as ms x ms, banded / all ms columns / the mmax columns that are there: m = 35, ms = 64
+// (h = 1/24, ell = 1.5, delta = 3) L = 64 561 / 82 / 83, L = 512 565 / 279 / 205, L = 2048 655 / 903 / 595; m = 47,
+// ms = 64 (ell = 2) L = 2048 848 / 904 / 699; m = 71, ms = 96 (ell = 3) L = 2048 3923 / 1943 / 1494.
 void block_groups(dd_ctx* c, int want) {
   const BlkGeo B = blk_geo(c);
   const int RG = B.ms / 32, N = c->g.nsub, sms = 152;
@@ -788,7 +795,8 @@ static void launch_cluster(void (*kern)(KArgs...), int blocks, int threads, size
 
 template <int P, int CR>
 static void launch_block_solve_t(dd_ctx* c, const BlkGeo& B, const double* r, cudaStream_t s) {
-  const BlkShape sh{c->blk_R, c->blk_PW, c->blk_RW, c->blk_rgl};
+  const int nch = (B.mmax + 8 * c->blk_PW - 1) / (8 * c->blk_PW);
+  const BlkShape sh{c->blk_R, c->blk_PW, c->blk_RW, c->blk_rgl, nch, 8 * nch};
   static PerDeviceOnce attr;
   once_per_device(attr, [] {
     DD_CUDA(cudaFuncSetAttribute(k_block_solve<P, CR>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
