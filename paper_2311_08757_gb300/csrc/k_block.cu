@@ -133,7 +133,7 @@ __global__ void k_schur_form(Geo g, BlkGeo B, const double* __restrict__ tabS, c
 //   J = I:   A(I, I) = P,  A(K, I) = -A(K, I) P          (P the inverse of A(I, I))
 //   J != I:  A(I, J) = P A(I, J) = U,  A(K, J) -= A(K, I) U
 constexpr int kGjThreads = 256;
-__global__ void __launch_bounds__(kGjThreads) k_gj_panel(BlkGeo B, const double* __restrict__ in,
+__global__ void __launch_bounds__(kGjThreads) k_gj_panel(Geo g, BlkGeo B, const double* __restrict__ in,
                                                          double* __restrict__ out, double* __restrict__ Sinv, int s,
                                                          int p, int* flag) {
   __shared__ double Pm[32][33], U[32][33], C[32][33];
@@ -149,7 +149,8 @@ __global__ void __launch_bounds__(kGjThreads) k_gj_panel(BlkGeo B, const double*
     U[r][col] = A[(size_t)(32 * p + r) * ms + 32 * jt + col];
   }
   __syncthreads();
-  for (int k = 0; k < 32; ++k) {
+  const int npiv = min(32, B.w2[c.ty] * g.nyi - 32 * p);   // pivots past m are rows of the identity
+  for (int k = 0; k < npiv; ++k) {
     if (r0 == 0) {
       double piv = Pm[k][k];
       if (!(piv > 0.0)) {
@@ -234,7 +235,7 @@ void block_factor(dd_ctx* c, int* flag) {
     if (g.p == 1) (k_schur_form<1><<<dim3(B.ms, chains), 128, smem, st>>>(g, B, c->tabS, c->blkS, s, half[0]), note_launch());
     else (k_schur_form<2><<<dim3(B.ms, chains), 128, smem, st>>>(g, B, c->tabS, c->blkS, s, half[0]), note_launch());
     for (int p = 0; p < np; ++p)
-      (k_gj_panel<<<dim3(np, chains), kGjThreads, 0, st>>>(B, half[p & 1], half[(p + 1) & 1], p + 1 == np ? c->blkS : nullptr,
+      (k_gj_panel<<<dim3(np, chains), kGjThreads, 0, st>>>(g, B, half[p & 1], half[(p + 1) & 1], p + 1 == np ? c->blkS : nullptr,
                                                            s, p, flag),
        note_launch());
   };
