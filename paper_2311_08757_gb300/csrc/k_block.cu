@@ -493,11 +493,19 @@ __global__ void __launch_bounds__(1024) k_block_solve(Geo g, BlkGeo B, BlkShape 
 // enough).  A plane's S^{-1} is one 8 KB block; a warp of its own brings the planes into a ring
 // by bulk copies ahead of their use.  f, h_k and (p = 1) the coupling coefficients are loaded two
 // planes ahead.  The two sides meet through one mbarrier per subdomain.
+//
+// TRIM (one warp per subdomain, planes of at most 28 unknowns): not past the plane's own columns
+// inside a group of four.  Long boxes of thin planes are bound by the pipe, and there the groups alone
+// cost more than the banded sweeps' single columns did.  us per launch, banded / groups / TRIM, L = 2048: 5
+// unknowns (n = 12) 40 / 56 / 44, 9 (n = 8) 44 / 50 / 42, 14 (n = 30) 191 / 202 / 170, 23 (n = 24) 249 / 223 / 198, 27
+// (n = 14) 153 / 135 / 122; the same up to L = 400.  29 unknowns and more have at most three columns to leave out: L = 400,
+// 31 (n = 32) 381 / 94 / 101, L = 2048 440 / 334 / 335.
 constexpr int ERR_BLK_WAIT = 1 << 8;   // error-word bit: a plane of S^{-1} or the other side did not arrive in time
 constexpr int row_stages(int PW) { return PW == 1 ? 3 : 6; }
 constexpr size_t row_smem(int PW) { return row_stages(PW) * 32 * 32 * sizeof(double); }
 
-template <int P, int PW>
+constexpr int kRowTrimMax = 28;
+template <int P, int PW, bool TRIM = false>
 __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_row(Geo g, BlkGeo B, const Sub* __restrict__ subs,
                                                          const int2* __restrict__ groups,
                                                          const int* __restrict__ sub_of_slot,
@@ -617,9 +625,9 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
           nv = ga[b / 2 + 3];
         }
         acc = fma(a0, u.x, acc);
-        acc = fma(a1, u.y, acc);
-        acc = fma(a2, v.x, acc);
-        acc = fma(a3, v.y, acc);
+        if (!TRIM || b + 1 < m) acc = fma(a1, u.y, acc);
+        if (!TRIM || b + 2 < m) acc = fma(a2, v.x, acc);
+        if (!TRIM || b + 3 < m) acc = fma(a3, v.y, acc);
         a0 = n0; a1 = n1; a2 = n2; a3 = n3;
         u = nu; v = nv;
       }
@@ -818,6 +826,7 @@ static void launch_block_solve_p(dd_ctx* c, const double* r, cudaStream_t s) {
       DD_CUDA(cudaFuncSetAttribute(k_block_solve_row<P, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
     });
     auto kern = c->blk_PW == 1 ? k_block_solve_row<P, 1> : (c->blk_PW == 2 ? k_block_solve_row<P, 2> : k_block_solve_row<P, 4>);
+    if (P == 1 && c->blk_PW == 1 && B.mmax <= kRowTrimMax) kern = k_block_solve_row<1, 1, true>;
     launch_cluster(kern, c->ngroups * 2, 32 * (c->blk_R * c->blk_PW + 1), row_smem(c->blk_PW), 2, s, c->g, B, (const Sub*)c->subs,
                    (const int2*)c->groups, (const int*)c->sub_of_slot, r, (const double*)c->tabS,
                    (const double*)c->blkS, c->Y64, c->kpad, (const PcgState*)c->st, c->dev_err + 8);
