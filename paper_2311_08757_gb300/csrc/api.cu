@@ -1430,8 +1430,8 @@ int dd_set_option(dd_ctx* c, int option, int value) {
       c->prolong_arith = (c->prolong_closed && !value) ? 1 : 0;
       break;
     case DD_OPT_GEMM_TILE_N:
-      if (value != 0 && value != 128 && value != 160 && value != 256)
-        return fail(c, DD_EINVAL, "GEMM tile N must be 0, 128, 160 or 256");
+      if (value != 0 && value != 64 && value != 128 && value != 160 && value != 256)
+        return fail(c, DD_EINVAL, "GEMM tile N must be 0, 64, 128, 160 or 256");
       c->gemm_bn_opt = value;
       break;
     case DD_OPT_LOCAL_RHS: {
