@@ -254,6 +254,8 @@ struct dd_ctx {
   double *stage_a = nullptr, *stage_b = nullptr;         // unpadded staging (ndof)
 
   // local solves
+  bool blk_glob = false;      // FP64: the solves' vectors in blk_vec (planes too large for shared memory)
+  double* blk_vec = nullptr;
   double* blkS = nullptr;     // FP64: [type][plane] inverse Schur complements of the local matrices
   float* bandCB32 = nullptr;  // mixed form: [type][nloc_max][band+1] column band of L (its inverse is rounded)
   float* bandRB32 = nullptr;  // [type][nloc_max][band+1] row band of L

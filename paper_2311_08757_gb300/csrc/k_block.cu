@@ -223,6 +223,7 @@ static BlkGeo blk_geo(const dd_ctx* c) {
 void block_factor(dd_ctx* c, int* flag) {
   const Geo& g = c->g;
   const BlkGeo B = blk_geo(c);
+  if (sizeof(double) * 2 * B.ms > 220 * 1024) throw Error(DD_EINVAL, "fixed direction too long for the FP64 local solves");
   const size_t blk = (size_t)B.ms * B.ms;
   cudaStream_t st = c->stream;
   if (!c->blkS) c->blkS = (double*)dev_alloc(c, sizeof(double) * blk * B.ntypes * B.kmax);
@@ -308,17 +309,26 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t a, uint32_t parity, i
   return false;
 }
 
-template <int P, int CR>
+// Planes of more than 7040 unknowns (three planes at most, the local vectors were bounded before) keep
+// the block's vectors in global memory (GLOB: 4 R ms doubles per block at `scratch`).
+template <int P, int CR, bool GLOB>
 __global__ void __launch_bounds__(1024) k_block_solve(Geo g, BlkGeo B, BlkShape sh, const Sub* __restrict__ subs,
                                                       const int2* __restrict__ groups,
                                                       const int* __restrict__ sub_of_slot,
                                                       const double* __restrict__ r, const double* __restrict__ tabS,
                                                       const double* __restrict__ Sinv, double* __restrict__ Y, int kpad,
-                                                      const PcgState* st) {
+                                                      const PcgState* st, double* scratch) {
   if (st != nullptr && st->done) return;
   cluster_arrive();   // waited for before the first store into another block's shared memory
-  extern __shared__ double sm[];
+  extern __shared__ double s_blk[];
   const unsigned rank = cluster_rank();
+  const size_t vlen = (size_t)4 * sh.R * B.ms;
+  double* const sm = GLOB ? scratch + blockIdx.x * vlen : s_blk;
+  // store to the same variable of block `to` of the cluster
+  auto remote = [&](double* local, unsigned to, double v) {
+    if (GLOB) local[((long long)to - (long long)rank) * (long long)vlen] = v;
+    else dsm_store(local, to, v);
+  };
   const int side = (int)rank / CR, cr = (int)rank % CR;
   const int2 grp = groups[blockIdx.x / (2 * CR)];
   const int ms = B.ms, R = sh.R;
@@ -333,7 +343,7 @@ __global__ void __launch_bounds__(1024) k_block_solve(Geo g, BlkGeo B, BlkShape 
   double* gv = sm + (size_t)rr * ms;
   double* hb[2] = {sm + (size_t)(R + rr) * ms, sm + (size_t)(2 * R + rr) * ms};
   double* ub = sm + (size_t)(3 * R + rr) * ms;
-  double* part = sm + (size_t)4 * R * ms + (size_t)rr * sh.PW * sh.rgl * 32;
+  double* part = (GLOB ? s_blk : sm + (size_t)4 * R * ms) + (size_t)rr * sh.PW * sh.rgl * 32;
   const int lane = tr & 31, w = tr >> 5, rw = w % sh.RW, pw = w / sh.RW;
   const int cpp = sh.cpp, nch = sh.nch;             // columns and 8-column chunks of this warp's range
   const int rg_first = cr * sh.rgl + rw, rg_end = min((cr + 1) * sh.rgl, ms >> 5);
@@ -391,7 +401,7 @@ __global__ void __launch_bounds__(1024) k_block_solve(Geo g, BlkGeo B, BlkShape 
     if (CR == 1) h[row] = v;
     else
 #pragma unroll
-      for (int q = 0; q < CR; ++q) dsm_store(h + row, side * CR + q, v);
+      for (int q = 0; q < CR; ++q) remote(h + row, side * CR + q, v);
   };
   auto ypos = [&](int k, int row) -> size_t {
     const int c2 = (P == 1) ? 0 : row / nyi;
@@ -435,7 +445,7 @@ __global__ void __launch_bounds__(1024) k_block_solve(Geo g, BlkGeo B, BlkShape 
       const int c2 = (P == 1) ? 0 : row / nyi;
       const double v = (row < m && nmine > 0)
                            ? blk_couple<P>(g, tabS, B, ty, t, c2, row - c2 * nyi, 1, hb[(nmine - 1) & 1]) : 0.0;
-      dsm_store(ub + row, cr, v);
+      remote(ub + row, cr, v);
     }
   cluster_sync_all();
   int cur = t & 1;   // the buffer that takes x_t: the left side has just read the other one
@@ -453,7 +463,7 @@ __global__ void __launch_bounds__(1024) k_block_solve(Geo g, BlkGeo B, BlkShape 
     if (nmine == 0 && rg_first < rg_end) load8(chunk0(t, rg_first));
     product(t, nmine > 0 ? t - 1 : -1, [&](int row, double v) {
 #pragma unroll
-      for (int q = 0; q < 2 * CR; ++q) dsm_store(hb[cur] + row, q, v);
+      for (int q = 0; q < 2 * CR; ++q) remote(hb[cur] + row, q, v);
       if (live && row < m) yb[ypos(t, row)] = v;
     });
   } else if (nmine > 0 && rg_first < rg_end) {
@@ -752,6 +762,7 @@ void block_groups(dd_ctx* c, int want) {
   const BlkGeo B = blk_geo(c);
   const int RG = B.ms / 32, N = c->g.nsub, sms = 152;
   int cr = 1, PW = 1, RW = 1, rgl = 1, R = 1;
+  bool glob = false;
   if (RG == 1) {
     PW = 8 * N <= 4 * sms ? 4 : (4 * N <= 8 * sms ? 2 : 1);
     const double x = 2.0 * N / (4 * sms);   // half chains per sub-partition
@@ -767,7 +778,7 @@ void block_groups(dd_ctx* c, int want) {
     while (R > 1 && R * RW * PW > 32) R /= 2;
     const size_t per = sizeof(double) * ((size_t)4 * B.ms + (PW > 1 ? (size_t)PW * rgl * 32 : 0));
     while (R > 1 && per * R > 200 * 1024) R /= 2;
-    if (per * R > 220 * 1024) throw Error(DD_EINVAL, "fixed direction too long for the FP64 local solves");
+    glob = per * R > 220 * 1024;
   }
   c->blk_cr = cr;
   c->blk_R = R;
@@ -779,6 +790,8 @@ void block_groups(dd_ctx* c, int want) {
     for (int j = 0; j < c->type_count[t]; j += R)
       grp.push_back(make_int2(c->type_first[t] + j, std::min(R, c->type_count[t] - j)));
   c->ngroups = (int)grp.size();
+  c->blk_glob = glob;   // R = 1 and cr = 4 then, whatever was asked for: allocated once
+  if (glob && !c->blk_vec) c->blk_vec = (double*)dev_alloc(c, sizeof(double) * 4 * B.ms * (size_t)grp.size() * 2 * cr);
   DD_CUDA(cudaMemcpyAsync(c->groups, grp.data(), sizeof(int2) * grp.size(), cudaMemcpyHostToDevice, c->stream));
   DD_CUDA(cudaStreamSynchronize(c->stream));   // grp is a temporary
 }
@@ -802,18 +815,18 @@ static void launch_cluster(void (*kern)(KArgs...), int blocks, int threads, size
   note_launch();
 }
 
-template <int P, int CR>
+template <int P, int CR, bool GLOB = false>
 static void launch_block_solve_t(dd_ctx* c, const BlkGeo& B, const double* r, cudaStream_t s) {
   const int nch = (B.mmax + 8 * c->blk_PW - 1) / (8 * c->blk_PW);
   const BlkShape sh{c->blk_R, c->blk_PW, c->blk_RW, c->blk_rgl, nch, 8 * nch};
   static PerDeviceOnce attr;
   once_per_device(attr, [] {
-    DD_CUDA(cudaFuncSetAttribute(k_block_solve<P, CR>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+    DD_CUDA(cudaFuncSetAttribute(k_block_solve<P, CR, GLOB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
   });
-  const size_t smem = sizeof(double) * sh.R * ((size_t)4 * B.ms + (sh.PW > 1 ? (size_t)sh.PW * sh.rgl * 32 : 0));
-  launch_cluster(k_block_solve<P, CR>, c->ngroups * 2 * CR, 32 * sh.R * sh.PW * sh.RW, smem, 2 * CR, s, c->g, B, sh,
+  const size_t smem = sizeof(double) * sh.R * ((GLOB ? 0 : (size_t)4 * B.ms) + (sh.PW > 1 ? (size_t)sh.PW * sh.rgl * 32 : 0));
+  launch_cluster(k_block_solve<P, CR, GLOB>, c->ngroups * 2 * CR, 32 * sh.R * sh.PW * sh.RW, smem, 2 * CR, s, c->g, B, sh,
                  (const Sub*)c->subs, (const int2*)c->groups, (const int*)c->sub_of_slot, r, (const double*)c->tabS,
-                 (const double*)c->blkS, c->Y64, c->kpad, (const PcgState*)c->st);
+                 (const double*)c->blkS, c->Y64, c->kpad, (const PcgState*)c->st, c->blk_vec);
 }
 
 template <int P>
@@ -830,6 +843,8 @@ static void launch_block_solve_p(dd_ctx* c, const double* r, cudaStream_t s) {
     launch_cluster(kern, c->ngroups * 2, 32 * (c->blk_R * c->blk_PW + 1), row_smem(c->blk_PW), 2, s, c->g, B, (const Sub*)c->subs,
                    (const int2*)c->groups, (const int*)c->sub_of_slot, r, (const double*)c->tabS,
                    (const double*)c->blkS, c->Y64, c->kpad, (const PcgState*)c->st, c->dev_err + 8);
+  } else if (c->blk_glob) {
+    launch_block_solve_t<P, 4, true>(c, B, r, s);
   } else if (c->blk_cr == 1) {
     launch_block_solve_t<P, 1>(c, B, r, s);
   } else if (c->blk_cr == 2) {
