@@ -28,9 +28,9 @@ namespace dd {
 constexpr int kBandWinMax = 160;
 
 __device__ __forceinline__ double rsqrt_el(double v) { return rsqrt(v); }
-__device__ __forceinline__ float rsqrt_el(float v) { return rsqrtf(v); }   // wide bands
+__device__ __forceinline__ float rsqrt_el(float v) { return rsqrtf(v); }
 
-// FP64 (the coarse matrix); FP32 factors take k_band_factor_panel
+// FP64 (the coarse matrix), and FP32 above the bands of k_band_factor_panel
 template <typename T, int P, int PPT>
 __global__ void __launch_bounds__(1024) k_band_factor_win(T* CB, T* inv, const int* __restrict__ nvec,
                                                           int nmax, int b, int* flag) {
@@ -89,21 +89,36 @@ __global__ void __launch_bounds__(1024) k_band_factor_win(T* CB, T* inv, const i
     for (int u = 0; u < P; ++u) {
       const int k = k0 + u;
       if (k < n) {
-        // one thread forms the pivot's reciprocal square root (the FP64 pipe would pay for
-        // every redundant copy)
-        if (t == 0) {
+        T il;
+        if constexpr (sizeof(T) == 4) {
+          // FP32: every thread forms the pivot's reciprocal square root itself (identical
+          // values), which saves the barrier that publishing it would take
           T piv = win[sk * S];
           if (!(piv > (T)0)) {
-            atomicOr(flag, 1);
+            if (t == 0) atomicOr(flag, 1);
             piv = (T)1;
           }
-          const T l = rsqrt_el(piv);
-          A[(size_t)k * bs] = piv * l;
-          iv[k] = l * l;
-          colk[0] = l;
+          il = rsqrt_el(piv);
+          if (t == 0) {
+            A[(size_t)k * bs] = piv * il;
+            iv[k] = il * il;
+          }
+        } else {
+          // FP64: one thread (the FP64 pipe would pay for every redundant copy)
+          if (t == 0) {
+            T piv = win[sk * S];
+            if (!(piv > (T)0)) {
+              atomicOr(flag, 1);
+              piv = (T)1;
+            }
+            const T l = rsqrt_el(piv);
+            A[(size_t)k * bs] = piv * l;
+            iv[k] = l * l;
+            colk[0] = l;
+          }
+          __syncthreads();
+          il = colk[0];
         }
-        __syncthreads();
-        const T il = colk[0];
         const int dmax = min(b, n - 1 - k);
         for (int d = 1 + t; d <= b; d += blockDim.x) {
           T v = (T)0;
@@ -141,7 +156,7 @@ __global__ void __launch_bounds__(1024) k_band_factor_win(T* CB, T* inv, const i
   cp_async_wait<0>();   // no copy into this block's shared memory outlives it
 }
 
-// FP32 factors of bands up to 160 (the local matrices of the mixed form, whose inverses are rounded
+// FP32 factors of bands up to 88 (the local matrices of the mixed form, whose inverses are rounded
 // to a tensor-core type, and the cell preconditioner): the same window and the same operations in
 // the same order (the same bits), eight columns at a time.  A column's chain (pivot, reciprocal
 // square root, scaling, update of the next column) with two block barriers bounds the rank-1 form at
@@ -150,10 +165,12 @@ __global__ void __launch_bounds__(1024) k_band_factor_win(T* CB, T* inv, const i
 // all eight to the trailing window with one read and write of each entry.  The columns that enter
 // are loaded a panel ahead.
 // Order 1209, band 32 (the three local types at L = 2048, n = 32): 549 -> 272 us; order 992, band 63
-// (its cell): 549 -> 316 us.
-constexpr int kPb = 8;
+// (its cell): 549 -> 316 us.  Wider bands keep the rank-1 form: the block's update (16 values read per entry
+// and panel) takes over there, and the panel's registers no longer fit beside blocks of more than 512
+// threads.  dd_coarse_build, n = 12, rank-1 / panels: band 88 2.11 / 1.74 ms, 89 2.12 / 2.37, 127 3.95 / 4.20, 160 11.5 / 12.2.
+constexpr int kPb = 8, kPanelBandMax = 88;
 template <int Q, int PPT>
-__global__ void __launch_bounds__(Q <= 3 ? 512 : 1024) k_band_factor_panel(float* CB, float* inv, const int* __restrict__ nvec,
+__global__ void __launch_bounds__(512) k_band_factor_panel(float* CB, float* inv, const int* __restrict__ nvec,
                                                             int nmax, int b, int* flag) {
   extern __shared__ __align__(16) unsigned char fsm_raw[];
   const int m = blockIdx.x;
@@ -426,7 +443,7 @@ template <typename T>
 static void factor_launch(T* CB, T* RB, T* inv, const int* nvec, int nmat, int nmax, int b, int* flag,
                           cudaStream_t s) {
   if (b <= kBandWinMax) {
-    size_t smem = sizeof(T) * ((size_t)(b + 1) * (((b + 1) + 1) & ~1) + (size_t)(b + 1) * (1 + 4));
+    const size_t smem = sizeof(T) * ((size_t)(b + 1) * (((b + 1) + 1) & ~1) + (size_t)(b + 1) * (1 + 4));
     // PPT triangle pairs per thread, the block at least one thread per entry of a column (the
     // window's entering columns are staged one entry per thread) and at most 1024 threads
     const int tot = b * (b + 1) / 2;
@@ -436,9 +453,10 @@ static void factor_launch(T* CB, T* RB, T* inv, const int* nvec, int nmat, int n
     int threads = ((tot + ppt - 1) / ppt + 31) / 32 * 32;
     threads = std::max(threads, (b + 1 + 31) / 32 * 32);
     threads = std::min(threads, 1024);
+    const bool panel = sizeof(T) == 4 && b <= kPanelBandMax;
     if constexpr (sizeof(T) == 4) {
       // one warp factors the panel; the block has a thread for a quarter of the entering values
-      threads = std::min(1024, std::max(threads, (2 * (b + 1) + 31) / 32 * 32));
+      if (panel) threads = std::min(1024, std::max(threads, (2 * (b + 1) + 31) / 32 * 32));
 #define DD_FPAN(Q_, PPT_)                                                                                          \
   do {                                                                                                             \
     static dd::PerDeviceOnce attr;   /* once per device and instance */                                            \
@@ -446,15 +464,16 @@ static void factor_launch(T* CB, T* RB, T* inv, const int* nvec, int nmat, int n
       DD_CUDA(cudaFuncSetAttribute(k_band_factor_panel<Q_, PPT_>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
                                    220 * 1024));                                                                   \
     });                                                                                                            \
-    smem = sizeof(float) * ((size_t)32 * Q_ * kPb + (size_t)(b + kPb) * ((b + 2) & ~1));                           \
-    (k_band_factor_panel<Q_, PPT_><<<nmat, threads, smem, s>>>(CB, inv, nvec, nmax, b, flag), dd::note_launch());   \
+    const size_t psm = sizeof(float) * ((size_t)32 * Q_ * kPb + (size_t)(b + kPb) * ((b + 2) & ~1));               \
+    (k_band_factor_panel<Q_, PPT_><<<nmat, threads, psm, s>>>(CB, inv, nvec, nmax, b, flag), dd::note_launch());    \
   } while (0)
-      if (b + kPb <= 64) DD_FPAN(2, 4);         // tot <= 1596
-      else if (ppt == 4) DD_FPAN(3, 4);         // b <= 63
-      else if (b + kPb <= 96) DD_FPAN(3, 8);    // b <= 88: 3916 entries
-      else DD_FPAN(6, 16);
+      if (panel) {
+        if (b + kPb <= 64) DD_FPAN(2, 4);       // tot <= 1596
+        else if (ppt == 4) DD_FPAN(3, 4);       // b <= 63
+        else DD_FPAN(3, 8);                     // b <= 88: 3916 entries
+      }
 #undef DD_FPAN
-    } else {
+    }
 #define DD_FWIN(PPT_)                                                                                         \
   do {                                                                                                      \
     static dd::PerDeviceOnce attr;   /* once per device and instance */                                     \
@@ -464,11 +483,12 @@ static void factor_launch(T* CB, T* RB, T* inv, const int* nvec, int nmat, int n
     });                                                                                                     \
     (k_band_factor_win<T, 4, PPT_><<<nmat, threads, smem, s>>>(CB, inv, nvec, nmax, b, flag), dd::note_launch()); \
   } while (0)
-    if (ppt == 4) DD_FWIN(4);
-    else if (ppt == 8) DD_FWIN(8);
-    else DD_FWIN(16);
-#undef DD_FWIN
+    if (!panel) {
+      if (ppt == 4) DD_FWIN(4);
+      else if (ppt == 8) DD_FWIN(8);
+      else DD_FWIN(16);
     }
+#undef DD_FWIN
   } else {
     const int np = std::min<int>(kPanel, (int)((200 * 1024) / (sizeof(T) * (size_t)(b + 1))));
     if (np < 1) throw Error(DD_EINVAL, "band too wide for the shared-memory panel factorisation");
