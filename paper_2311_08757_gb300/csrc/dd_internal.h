@@ -254,6 +254,7 @@ struct dd_ctx {
   double *stage_a = nullptr, *stage_b = nullptr;         // unpadded staging (ndof)
 
   // local solves
+  bool blk_half = false;      // FP64: a warp takes two subdomains
   bool blk_glob = false;      // FP64: the solves' vectors in blk_vec (planes too large for shared memory)
   double* blk_vec = nullptr;
   double* blkS = nullptr;     // FP64: [type][plane] inverse Schur complements of the local matrices

@@ -504,25 +504,29 @@ __global__ void __launch_bounds__(1024) k_block_solve(Geo g, BlkGeo B, BlkShape 
 // by bulk copies ahead of their use.  f, h_k and (p = 1) the coupling coefficients are loaded two
 // planes ahead.  The two sides meet through one mbarrier per subdomain.
 //
-// TRIM (one warp per subdomain, planes of at most 28 unknowns): not past the plane's own columns
-// inside a group of four.  Long boxes of thin planes are bound by the pipe, and there the groups alone
-// cost more than the banded sweeps' single columns did.  us per launch, banded / groups / TRIM, L = 2048: 5
-// unknowns (n = 12) 40 / 56 / 44, 9 (n = 8) 44 / 50 / 42, 14 (n = 30) 191 / 202 / 170, 23 (n = 24) 249 / 223 / 198, 27
-// (n = 14) 153 / 135 / 122; the same up to L = 400.  29 unknowns and more have at most three columns to leave out: L = 400,
-// 31 (n = 32) 381 / 94 / 101, L = 2048 440 / 334 / 335.
+// With one warp per subdomain the FP64 pipe bounds long boxes, and thin planes leave most of it to
+// padding; there the form above cost more than the banded sweeps it replaced.
+// TRIM (planes of at most 28 unknowns): the products end at the plane's own columns, inside a group of
+// four.  us per launch at L = 2048, banded / groups of four / TRIM: 19 unknowns (n = 20) 170 / 157 / 137, 23 (n = 24)
+// 249 / 223 / 198, 27 (n = 14) 153 / 135 / 122; the same at L = 400.  29 unknowns and more have at most three columns to
+// leave out: 31 (n = 32) 440 / 334 / 335, at L = 400 381 / 94 / 101.
+// HALF (planes of at most 16 unknowns, TRIM too): a warp takes two subdomains, each half of it one's rows, so
+// every instruction works for both; the pair reads the same S^{-1}.  us per launch, banded / TRIM / HALF: 15 unknowns
+// (n = 16) L = 310 99 / 36 / 35, L = 2048 113 / 97 / 58, L = 8000 371 / 344 / 193; 5 (n = 12) L = 4000 60 / 82 / 47; 3 (n = 4)
+// L = 20000 111 / 135 / 83.
 constexpr int ERR_BLK_WAIT = 1 << 8;   // error-word bit: a plane of S^{-1} or the other side did not arrive in time
 constexpr int row_stages(int PW) { return PW == 1 ? 3 : 6; }
 constexpr size_t row_smem(int PW) { return row_stages(PW) * 32 * 32 * sizeof(double); }
 
-constexpr int kRowTrimMax = 28;
-template <int P, int PW, bool TRIM = false>
+constexpr int kRowTrimMax = 28, kRowHalfMax = 16;
+template <int P, int PW, bool TRIM = false, bool HALF = false>
 __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_row(Geo g, BlkGeo B, const Sub* __restrict__ subs,
                                                          const int2* __restrict__ groups,
                                                          const int* __restrict__ sub_of_slot,
                                                          const double* __restrict__ r, const double* __restrict__ tabS,
                                                          const double* __restrict__ Sinv, double* __restrict__ Y,
                                                          int kpad, const PcgState* st, int* err) {
-  constexpr int CPP = 32 / PW, MS = 32, NT = (P == 1) ? 3 : 9, D = row_stages(PW);
+  constexpr int CPP = HALF ? 16 : 32 / PW, MS = 32, NT = (P == 1) ? 3 : 9, D = row_stages(PW);
   if (st != nullptr && st->done) return;
   extern __shared__ __align__(128) double s_ring[];  // [D][32][32]
   __shared__ __align__(16) double s_g[4][32];        // per warp: the product's argument
@@ -551,14 +555,15 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
   cluster_wait();
   if (w == nw) {   // the ring's producer
     if (lane == 0) {
+      // the columns that the shares cover, in whole groups of four
+      const uint32_t bytes = PW * (((B.w2[ty] * g.nyi + PW - 1) / PW + 3) & ~3) * MS * sizeof(double);
       int q = 0;
       for (; q < nprod; ++q) {
         const int sl = q % D;
         if (q >= D && !mbar_wait(bar + 8 * (D + sl), (uint32_t)(q / D - 1) & 1u, err, ERR_BLK_WAIT)) break;
         const int i = q < nmine ? q : 2 * nmine - q - (side ? 1 : 0);   // plane i from this side's end (nmine: t)
-        mbar_expect_tx(bar + 8 * sl, MS * MS * sizeof(double));
-        bulk_g2s(smem_u32(s_ring + sl * MS * MS), blk_inverse(B, Sinv, ty, k0 + dir * i), MS * MS * sizeof(double),
-                 bar + 8 * sl);
+        mbar_expect_tx(bar + 8 * sl, bytes);
+        bulk_g2s(smem_u32(s_ring + sl * MS * MS), blk_inverse(B, Sinv, ty, k0 + dir * i), bytes, bar + 8 * sl);
       }
       // the last copy into each slot: a warp that gave up has not waited for it
       for (int k = max(0, q - D); k < q; ++k) mbar_wait(bar + 8 * (k % D), (uint32_t)(k / D) & 1u, err, ERR_BLK_WAIT);
@@ -566,13 +571,15 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
     cluster_sync_all();
     return;
   }
-  const int rr = w / PW, pw = w % PW;
+  const int ws = w / PW, pw = w % PW;                // the warps of one subdomain (HALF: of a pair of them)
+  const int half = HALF ? lane & 16 : 0, row = lane - half;
+  const int rr = HALF ? 2 * ws + (half >> 4) : ws;
   const bool live = rr < grp.y;
   const Sub sb = subs[sub_of_slot[grp.x + (live ? rr : 0)]];
   const int w2 = B.w2[ty], nyi = g.nyi, m = w2 * nyi;
   const int cpp = ((m + PW - 1) / PW + 3) & ~3;      // columns of this warp's share (S and g are 0 past m)
-  const bool in = lane < m;
-  const int c2 = (P == 1) ? 0 : lane / nyi, sj = lane - c2 * nyi;
+  const bool in = row < m;
+  const int c2 = (P == 1) ? 0 : row / nyi, sj = row - c2 * nyi;
   const long long cstride = (P == 1) ? g.Ypad : (long long)g.ncx * g.Ypad;
   const double* rb = r + ((P == 1) ? (long long)sb.lo1 * g.Ypad : ((long long)sb.lo1 * g.ncx + sb.lo2) * g.Ypad) +
                      (long long)c2 * g.Ypad + sj;
@@ -601,22 +608,22 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
 #pragma unroll
     for (int e = 0; e < NT; ++e) {
       const int off = (P == 1) ? e - 1 : (e / 3 - 1) * nyi + e % 3 - 1;
-      hn[e] = __shfl_sync(kFull, h, (lane + off) & 31);
+      hn[e] = __shfl_sync(kFull, h, HALF ? half + ((row + off) & 15) : (lane + off) & 31);
     }
 #pragma unroll
     for (int e = 0; e < NT; ++e) v = fma(-cf[e], hn[e], v);
     return v;
   };
   int buf = 0, q = 0, sl = 0, ph = 0;   // product q reads ring slot sl at parity ph
-  // init + S_k^{-1} g (row `lane`) for the next plane in turn
+  // init + S_k^{-1} g (this lane's row) for the next plane in turn
   auto product = [&](double gl, double init) -> double {
     double* gs = s_g[w];
     __syncwarp();
     gs[lane] = gl;
     __syncwarp();
     wait(bar + 8 * sl, (uint32_t)ph);
-    const double* Sp = s_ring + sl * MS * MS + pw * cpp * MS + lane;
-    const double2* ga = reinterpret_cast<const double2*>(gs + pw * cpp);
+    const double* Sp = s_ring + sl * MS * MS + pw * cpp * MS + row;
+    const double2* ga = reinterpret_cast<const double2*>(gs + half + pw * cpp);
     double acc = init;
     // four columns at a time, the next four loaded beside them
     double a0 = Sp[0], a1 = Sp[MS], a2 = Sp[2 * MS], a3 = Sp[3 * MS];
@@ -650,10 +657,10 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
       ph ^= 1;
     }
     if (PW == 1) return acc;
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + rr), "n"(32 * PW) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + ws), "n"(32 * PW) : "memory");
     double p[PW];
 #pragma unroll
-    for (int j = 0; j < PW; ++j) p[j] = s_part[buf][rr * PW + j][lane];
+    for (int j = 0; j < PW; ++j) p[j] = s_part[buf][ws * PW + j][lane];
     acc = p[0];
 #pragma unroll
     for (int j = 1; j < PW; ++j) acc += p[j];
@@ -688,15 +695,15 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
     }
   }
   // ---- plane t: the right side's first warp sends its coupling, the left side's x_t
-  const uint32_t meet = bar + 8 * (2 * D + rr);
+  const uint32_t meet = bar + 8 * (2 * D + ws);
   auto send = [&](double v) {
     if (pw != 0) return;
-    dsm_store(&s_mid[rr][lane], side ^ 1, v);
+    dsm_store(&s_mid[ws][lane], side ^ 1, v);
     dsm_arrive(meet, side ^ 1);
   };
   auto receive = [&]() -> double {
     if (!dead && !mbar_wait_cluster(meet, 0, err, ERR_BLK_WAIT)) dead = true;
-    return s_mid[rr][lane];
+    return s_mid[ws][lane];
   };
   if (side == 1) send(nmine > 0 ? gl : 0.0);
   // h_k is read back by the warp that stored it
@@ -745,7 +752,7 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
 // L = 301 48 / 43 / 79, L = 350 49 / 76 / 78; h = 1/12, L = 200 24 / 22 / 30).  With PW = 1 the
 // blocks take 1, 2 or 4 subdomains: small blocks spread evenly over few rounds (us per launch for
 // 1 / 2 / 4 at h = 1/32: L = 512 88 / 96 / 96, L = 1000 187 / 158 / 177, L = 2048 361 / 353 / 319,
-// where four warps also share each plane's copy).
+// where four warps also share each plane's copy); pairs of subdomains per warp (HALF) by the same rule.
 // Larger planes (k_block_solve): a warp per 32 rows, up to 4 subdomains and 32 warps per block, up to 4 column
 // ranges while that leaves an SM sub-partition at most 5 warps, up to 4 blocks per side while the grid
 // does not fill the SMs.  The results do not depend on the subdomains per block.
@@ -762,11 +769,13 @@ void block_groups(dd_ctx* c, int want) {
   const BlkGeo B = blk_geo(c);
   const int RG = B.ms / 32, N = c->g.nsub, sms = 152;
   int cr = 1, PW = 1, RW = 1, rgl = 1, R = 1;
-  bool glob = false;
+  bool glob = false, half = false;
   if (RG == 1) {
     PW = 8 * N <= 4 * sms ? 4 : (4 * N <= 8 * sms ? 2 : 1);
-    const double x = 2.0 * N / (4 * sms);   // half chains per sub-partition
-    R = std::min(want > 0 ? want : (x <= 2.0 ? 1 : (x <= 5.0 ? 2 : 4)), 4 / PW);
+    half = c->g.p == 1 && PW == 1 && B.mmax <= kRowHalfMax;
+    const int pair = half ? 2 : 1;                     // subdomains per warp
+    const double x = 2.0 * N / (4 * sms * pair);       // warps with a half chain per sub-partition
+    R = std::min(want > 0 ? want : pair * (x <= 2.0 ? 1 : (x <= 5.0 ? 2 : 4)), pair * 4 / PW);
   } else {
     while (cr < 4 && 2 * cr <= RG && (long long)2 * N * cr * 2 <= sms) cr *= 2;
     while (cr < 4 && (RG + cr - 1) / cr > 32) cr *= 2;
@@ -790,6 +799,7 @@ void block_groups(dd_ctx* c, int want) {
     for (int j = 0; j < c->type_count[t]; j += R)
       grp.push_back(make_int2(c->type_first[t] + j, std::min(R, c->type_count[t] - j)));
   c->ngroups = (int)grp.size();
+  c->blk_half = half;
   c->blk_glob = glob;   // R = 1 and cr = 4 then, whatever was asked for: allocated once
   if (glob && !c->blk_vec) c->blk_vec = (double*)dev_alloc(c, sizeof(double) * 4 * B.ms * (size_t)grp.size() * 2 * cr);
   DD_CUDA(cudaMemcpyAsync(c->groups, grp.data(), sizeof(int2) * grp.size(), cudaMemcpyHostToDevice, c->stream));
@@ -839,8 +849,10 @@ static void launch_block_solve_p(dd_ctx* c, const double* r, cudaStream_t s) {
       DD_CUDA(cudaFuncSetAttribute(k_block_solve_row<P, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
     });
     auto kern = c->blk_PW == 1 ? k_block_solve_row<P, 1> : (c->blk_PW == 2 ? k_block_solve_row<P, 2> : k_block_solve_row<P, 4>);
-    if (P == 1 && c->blk_PW == 1 && B.mmax <= kRowTrimMax) kern = k_block_solve_row<1, 1, true>;
-    launch_cluster(kern, c->ngroups * 2, 32 * (c->blk_R * c->blk_PW + 1), row_smem(c->blk_PW), 2, s, c->g, B, (const Sub*)c->subs,
+    if (c->blk_half) kern = k_block_solve_row<1, 1, true, true>;
+    else if (P == 1 && c->blk_PW == 1 && B.mmax <= kRowTrimMax) kern = k_block_solve_row<1, 1, true>;
+    const int warps = c->blk_half ? (c->blk_R + 1) / 2 : c->blk_R * c->blk_PW;
+    launch_cluster(kern, c->ngroups * 2, 32 * (warps + 1), row_smem(c->blk_PW), 2, s, c->g, B, (const Sub*)c->subs,
                    (const int2*)c->groups, (const int*)c->sub_of_slot, r, (const double*)c->tabS,
                    (const double*)c->blkS, c->Y64, c->kpad, (const PcgState*)c->st, c->dev_err + 8);
   } else if (c->blk_glob) {
