@@ -330,8 +330,8 @@ int dd_apply_operator(dd_ctx* ctx, int op, const double* x, double* y);
 /* y = A_sigma x evaluated by the float-pair pass of the PCG iteration (DD_OPT_PAIRS: each
  * coefficient and x value split into two floats, error-free products and sums on the FP32
  * pipe, y = hi + lo in FP64), whatever DD_OPT_PAIRS is set to: p = 1 the fused p-update pass
- * with beta = 0, p = 2 the split p update and the pair matvec (by DD_OPT_TILED3).  It exposes that arithmetic for checking against dd_apply_operator
- * (DD_OP_ASIGMA).  Per node, |y_pairs - y| relative to the sum of |a_ij x_j| over the row: the
+ * with beta = 0, p = 2 the split p update and the pair matvec (by DD_OPT_TILED3).  It exposes
+ * that arithmetic for checking against dd_apply_operator (DD_OP_ASIGMA).  Per node, |y_pairs - y| relative to the sum of |a_ij x_j| over the row: the
  * splits and the dropped lo * lo product leave 2.5 * 2^-47 of each term; the FP32 roundings of
  * the low-order accumulator add an amount that grows with the number of taps.  Largest ratios
  * measured: 8.5 * 2^-47 with the 9 taps of p = 1, 13.4 * 2^-47 with the 27 of p = 2 (tested
@@ -416,8 +416,9 @@ int dd_coarse_matrix(dd_ctx* ctx, double* A0_host);
  *                       registers (each block takes the planes of one residue a1 mod n and the
  *                       same columns of every cell, so a thread keeps one class) and the split p
  *                       of three planes copied to shared memory, where Ypad <= 64; 0 reads the
- *                       table and p through the caches.  The same q; (p, q) summed in another
- *                       order [1]
+ *                       table and p through the caches; -1: as 1 for boxes large enough (about
+ *                       0.3M padded nodes at n Ypad = 128, 1.4M at 56), else as 0.  The same q;
+ *                       (p, q) summed in another order [-1]
  *   DD_OPT_X_LAG        1: the PCG update x_{k+1} = x_k + alpha_k p_k is made by iteration k + 1's
  *                       p update (which reads p_k anyway), and once more after the last
  *                       iteration, so the x/r update streams only r and q; the same FMA on the

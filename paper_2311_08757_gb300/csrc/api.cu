@@ -1406,7 +1406,7 @@ int dd_set_option(dd_ctx* c, int option, int value) {
       c->fuse_xr = value > 0 ? 1 : 0;
       break;
     case DD_OPT_TILED3:
-      if (value != 0 && value != 1) return fail(c, DD_EINVAL, "tiled p = 2 matvec must be 0 or 1");
+      if (value < -1 || value > 1) return fail(c, DD_EINVAL, "tiled p = 2 matvec must be -1, 0 or 1");
       c->matvec_tiled = value;
       break;
     case DD_OPT_X_LAG:

@@ -174,7 +174,7 @@ struct dd_ctx {
   int4 ptypes = {0, 0, 0, 0};       // p = 1: type ids of the left end, interior and right end subdomains
   int pdl = 0;                      // PCG chain kernels launched with programmatic dependent launch
   int fuse_xr_opt = -1;             // x/r update fused into the packing: 1 on, 0 off, -1 by the number of subdomains
-  int matvec_tiled = 1;             // p = 2 float pairs: the register-table matvec where it fits
+  int matvec_tiled = -1;            // p = 2 float pairs, the register-table matvec: 1 where it fits, 0 off, -1 by size
   // x_{k+1} = x_k + alpha_k p_k deferred to iteration k + 1's p update, which reads p_k anyway,
   // and one final update after the last iteration: the x/r update then streams r and q only
   int x_lag = 1;

@@ -965,7 +965,7 @@ __global__ void __launch_bounds__(kThreads) k_pupdate_pairs_cls(Geo g, int H, un
   }
 }
 
-bool matvec_cls_shape(const Geo& g, int* CW, int* ncg);
+bool matvec_cls(const dd_ctx* c, int* CW, int* ncg);
 
 // float2 elements of the split p: the padded vector, or the interleaved planes where those are longer
 long long split_p_len(const Geo& g) {
@@ -975,7 +975,7 @@ long long split_p_len(const Geo& g) {
 void launch_pupdate_pairs(dd_ctx* c, cudaStream_t s) {
   const long long n = c->g.plen;
   int CW = 0, ncg = 0;
-  if (c->matvec_tiled && matvec_cls_shape(c->g, &CW, &ncg)) {
+  if (matvec_cls(c, &CW, &ncg)) {
     const int H = cls_half(c->g);
     const unsigned total = (unsigned)((long long)c->g.ncx * (H + 2) * (c->g.Ypad / 2));   // below 2^31: two per node
     launch_chain(k_pupdate_pairs_cls, dim3(grid_blocks(total, kThreads)), dim3(kThreads), 0, s, c->pdl != 0, c->g, H,
@@ -1232,8 +1232,8 @@ __global__ void __launch_bounds__(kClsThreads, 3) k_matvec_pq_pairs_cls(Geo g, c
 }
 
 // column groups of the register-table form: the cell's n columns in ncg groups of CW, CW Ypad
-// threads each; Ypad at most 64 (the copies start one column before the vector, inside its guard band)
-bool matvec_cls_shape(const Geo& g, int* CW, int* ncg) {
+// threads each; Ypad at most 64 (two columns per block at least)
+static bool matvec_cls_shape(const Geo& g, int* CW, int* ncg) {
   const int most = kClsThreads / g.Ypad;
   if (g.p != 2 || most < 2) return false;
   *ncg = (g.n + most - 1) / most;
@@ -1241,11 +1241,25 @@ bool matvec_cls_shape(const Geo& g, int* CW, int* ncg) {
   return (long long)g.n * *ncg <= kMaxRedBlocks;   // one block per plane residue and group at least
 }
 
+// Whether the PCG takes the register-table form.  Without the option, where the box has enough nodes for
+// its blocks and a cell enough classes (n Ypad) for a block's threads; below that the cached form is
+// the faster one.  us per PCG iteration (BF16, delta = 1), cached / register table: n = 4, L = 64 (16 classes, 0.26M nodes) 92 /
+// 113; n = 8, ell = 0.5 (32) L = 24 (0.15M) 42 / 52, L = 64 (1.1M) 130 / 142, L = 100 (2.6M) 370 / 368; n = 6 (48) L = 64 (1.2M) 141 /
+// 142, L = 100 (2.9M) 388 / 382; n = 8 (64) L = 28 (0.41M) 59.7 / 61.1, L = 34 (0.60M) 70.6 / 69.6, L = 64 (2.1M) 180 / 164; n = 16, ell =
+// 0.5 (128) L = 8 (0.13M) 64.9 / 65.5, L = 12 (0.30M) 76.6 / 75.3; n = 12 (192) L = 10 (0.23M) 79 / 81, L = 14 (0.46M) 93 / 92; n = 16
+// (256) L = 6 (0.15M) 131 / 132, L = 24 (2.4M) 258 / 208.
+bool matvec_cls(const dd_ctx* c, int* CW, int* ncg) {
+  const Geo& g = c->g;
+  if (c->matvec_tiled == 0 || !matvec_cls_shape(g, CW, ncg)) return false;
+  const double nodes = (double)g.plen, cls = (double)g.n * g.Ypad;
+  return c->matvec_tiled > 0 || (nodes >= 262144.0 && nodes * cls >= (cls < 56.0 ? 80e6 : 36e6));
+}
+
 void launch_matvec_pq_pairs(dd_ctx* c, cudaStream_t s) {
   const Geo& g = c->g;
   if (g.p != 2) throw Error(DD_EINVAL, "the float-pair matvec pass is the p = 2 form");
   int CW = 0, ncg = 0;
-  if (c->matvec_tiled && matvec_cls_shape(g, &CW, &ncg)) {
+  if (matvec_cls(c, &CW, &ncg)) {
     const int threads = (CW * g.Ypad + 31) / 32 * 32;
     const size_t smem = sizeof(float4) * kClsStages * kClsPairs * (size_t)cls_cell_len(CW, g.Ypad);
     static PerDeviceOnce attr;
