@@ -568,7 +568,6 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
       // the last copy into each slot: a warp that gave up has not waited for it
       for (int k = max(0, q - D); k < q; ++k) mbar_wait(bar + 8 * (k % D), (uint32_t)(k / D) & 1u, err, ERR_BLK_WAIT);
     }
-    cluster_sync_all();
     return;
   }
   const int ws = w / PW, pw = w % PW;                // the warps of one subdomain (HALF: of a pair of them)
@@ -739,9 +738,11 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
       load_cf(pl(max(i - 1, 0)), dir, c1);
     }
   }
-  // On every path, also after a wait that gave up (its warp runs through the remaining, meaningless work
-  // without waiting): the other block's stores into this one have landed before it ends.
-  cluster_sync_all();
+  // A thread that has seen the meeting complete knows that the other block stores no more into this one.
+  // One whose wait gave up (it ran through the remaining, meaningless work without waiting) keeps the
+  // block alive until every thread of the other has ended or is here too (ended threads count as
+  // arrived); a barrier for all on every path cost 2% at L = 2048.
+  if (dead) cluster_sync_all();
 }
 
 // The launch shape.  Planes of at most 32 unknowns: PW warps per subdomain and side, 4 while every
