@@ -312,9 +312,9 @@ int stage_err(dd_ctx* c, int need) {
 bool use_gemm(const dd_ctx* c) { return c->grid.precision != DD_PREC_FP64; }
 
 // z = M^{-1} r on device padded vectors; mode 0 standalone, 1 PCG start, 2 PCG iteration.
-// The coarse right-hand side is formed in the pass that gathers R_i r (local solve or pack);
-// with tensor-core local solves the coarse solve then runs on a second stream beside the
-// GEMM (the two-level operator is additive, so the branches are independent).
+// The two-level operator is additive, so its branches are independent: the coarse solve runs on a
+// second stream beside the local solves.  Its right-hand side is formed in the packing of the
+// tensor-core form, and by a kernel of its own on that stream in FP64.
 // packed: the restrictions were packed by launch_pack_xr (a fused iteration), whose r update
 // the prolong-sum then applies.
 void precond(dd_ctx* c, const double* r, int mode, double* zout = nullptr, bool packed = false) {
@@ -1436,7 +1436,7 @@ int dd_set_option(dd_ctx* c, int option, int value) {
       break;
     case DD_OPT_LOCAL_RHS: {
       if (value != 0 && value != 1 && value != 2 && value != 4)
-        return fail(c, DD_EINVAL, "local right-hand sides per warp must be 0, 1, 2 or 4");
+        return fail(c, DD_EINVAL, "local right-hand sides per block must be 0, 1, 2 or 4");
       try {
         if (c->grid.precision == DD_PREC_FP64) block_groups(c, value);
       } catch (const Error& e) {

@@ -759,10 +759,10 @@ __global__ void __launch_bounds__(160, P == 1 && PW == 1 ? 7 : 3) k_block_solve_
 // does not fill the SMs.  The results do not depend on the subdomains per block.
 //
 // Measured against the banded triangular sweeps this replaced (one warp per one or two
-// subdomains, 2 n_loc dependent steps; us per application): p = 1, h = 1/32, delta = 4: L = 32
-// 375 -> 36, L = 512 376 -> 88, L = 2048 434 -> 319 (the FP64 pipe needs 288 for its instructions);
-// ell = 2, L = 300 1327 -> 209; p = 2, h = 1/16, delta = 2 (planes of 285): L = 6 5667 -> 292,
-// L = 16 5689 -> 1604 (pipe floor of the banded flops 1330).
+// subdomains, 2 n_loc dependent steps; us per application by events, the coarse branch beside it): p = 1,
+// h = 1/32, delta = 4: L = 37 375 -> 41, L = 512 390 -> 98, L = 2048 440 -> 328 (295 in the trace of a solve; the
+// FP64 pipe needs 288 for its instructions); ell = 2, L = 301 1335 -> 216; p = 2, h = 1/16, delta = 2 (planes of
+// 285): L = 6 5678 -> 298 (204 in a solve), L = 16 5689 -> 1604 (pipe floor of the banded flops 1330).
 // Planes of m unknowns stored as ms x ms, banded / all ms columns / the mmax columns that are there: m = 35, ms = 64
 // (h = 1/24, ell = 1.5, delta = 3) L = 64 561 / 82 / 83, L = 512 565 / 279 / 205, L = 2048 655 / 903 / 595; m = 47,
 // ms = 64 (ell = 2) L = 2048 848 / 904 / 699; m = 71, ms = 96 (ell = 3) L = 2048 3923 / 1943 / 1494.

@@ -1050,7 +1050,7 @@ __global__ void __launch_bounds__(kThreads) k_matvec_pq_pairs(Geo g, const float
 // summed in another order.
 //
 // L = 64, h = 1/16 (17M padded nodes), per launch in a solve: 232 us with the split p node by node (two
-// 8-byte loads and the moves that pair their halves for every tap of two nodes), 193 us as it is; the
+// 8-byte loads and the moves that pair their halves for every tap of two nodes), 193 to 197 us as it is; the
 // FP32 pipe needs 146 us for its 27 x 13 packed operations per two nodes, the copies 134 + 3.4 x 134 MB
 // mostly from L2.  The p update that writes the interleaved form: 94 us against 97.
 constexpr int kClsThreads = 128;
